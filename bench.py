@@ -191,18 +191,19 @@ def blas_threads():
 def kernel_model(name, n, steps, K):
     """(bound, algorithmic units per launch, unit kind, useful launches in K solves).
 
-    Algorithmic work: a transform along direction d costs 2 n_d flop per point
-    (FP64 path) or 3 split products = 6 n_d flop per point on the tensor cores
-    (mixed path); the bytes are one read of the input and one write of the
+    Algorithmic work: a transform along direction d costs 36 digit products = 72
+    n_d flop per point (FP64 path) or 3 split products = 6 n_d flop per point
+    (mixed path) on the tensor cores; the bytes are one read of the input and one write of the
     output field (FP32 intermediates, FP64 user arrays, 8-byte double-float
     solution).  Refinement rounds after convergence return at once and are not
     counted as useful launches."""
     P = float(n[0] * n[1] * n[2])
     rounds = 1 + steps
     t = {
-        # FP64 path: fwd and back transform of a direction share a name
-        "transform_x_f64": ("alu", 2.0 * P * n[0], "flop", 2 * rounds * K),
-        "transform_y_f64": ("alu", 2.0 * P * n[1], "flop", 2 * rounds * K),
+        # FP64 path: fwd and back transform of a direction share a name (digit
+        # products on the tensor cores, FP64 fields in and out)
+        "transform_x_f64": ("hbm", 16.0 * P, "byte", 2 * rounds * K),
+        "transform_y_f64": ("hbm", 16.0 * P, "byte", 2 * rounds * K),
         "thomas_z_f64": ("hbm", 16.0 * P, "byte", rounds * K),
         "residual_f64": ("hbm", 24.0 * P, "byte", rounds * K),
         # mixed path (bytes; the tensor flops are reported beside them)
@@ -227,6 +228,8 @@ def kernel_model(name, n, steps, K):
 def tensor_flops(name, n):
     P = float(n[0] * n[1] * n[2])
     d = {"x": 0, "y": 1, "z": 2}.get(name[len("transform_"):][:1], 1)
+    if name in ("transform_x_f64", "transform_y_f64"):
+        return 72.0 * P * n[d]  # 36 digit products
     return 6.0 * P * n[d] if name.endswith("_tc") else None
 
 

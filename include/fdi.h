@@ -75,7 +75,8 @@ typedef enum { FDI_BC_DIRICHLET = 0, FDI_BC_NEUMANN = 1 } fdi_bc;
 typedef enum { FDI_GRID_CELL = 0, FDI_GRID_MAC = 1 } fdi_grid;
 
 /* Arithmetic of the x/y eigenvector transforms (the dense contractions of
- * Eq. 25/29).  FDI_PREC_FP64: every step in FP64.  The mixed modes split each
+ * Eq. 25/29).  FDI_PREC_FP64: every step in FP64 (the transforms as exact
+ * products of 62-bit fixed-point digits, rounded to FP64 once).  The mixed modes split each
  * operand into a high and a low part in a 16-bit (or TF32) tensor-core type,
  * form hi*hi + hi*lo + lo*hi with FP32 accumulation, keep the intermediate
  * fields in FP32, run the Thomas sweep in FP32, and recover FP64 accuracy by
@@ -285,7 +286,8 @@ fdi_status fdi_eigen_noalloc(const double* faces, int n, int face_kind, fdi_bc b
  * until the next call of this function clears it.  The solution of a solve
  * that timed out is undefined.  Synchronises the device (the flag is cleared
  * once nothing runs); drops the plan's captured graphs.  FP64 plans accept
- * the call and have no such waits.  cycles < 0: FDI_ERR_INVALID_ARG. */
+ * the call; the waits inside their transforms keep the default bound.
+ * cycles < 0: FDI_ERR_INVALID_ARG. */
 fdi_status fdi_plan_set_wait_limit(fdi_plan* plan, long long cycles);
 
 /* Resident solve of mixed plans (enable = 1; default 0): a field whose x

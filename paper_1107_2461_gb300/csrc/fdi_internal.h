@@ -46,6 +46,9 @@ struct Axis {
   // mixed-precision data of this operator (tensor-core matrices, FP32 and
   // double-float coefficients); owned, see mixed.cu
   void* mixed = nullptr;
+  // FP64 plans: digit planes of E and E^{-1} for the tensor-core transforms of
+  // the directions that are transformed; owned, see slice_transform.cu
+  void* slices = nullptr;
   // host copies
   std::vector<double> h_m, h_kd, h_ko;
 };
@@ -315,11 +318,11 @@ fdi_status eigen_decompose_batch(int count, int n, const double* m, const double
                                  bool zero_flux0, double* lam_all, double* E_all, double* Einv_all, cudaStream_t s,
                                  int* d_err);
 
-// FP64 path launchers (kernels_f64.cu)
-fdi_status launch_lines_f64(fdi_plan* p, const double* in, double* out, const double* T, int nin,
-                            int nout, long long lines, bool accumulate, const int* skip, cudaStream_t s);
-fdi_status launch_slab_f64(fdi_plan* p, const double* in, double* out, const double* T, int nin,
-                           int nout, long long ncols, int batch, const int* skip, cudaStream_t s);
+// FP64 path launchers (kernels_f64.cu).  Transform of direction d of a field by
+// E_d^{-1} (forward) or E_d: out (+)= T in along every line of d (x lines may
+// accumulate), on the tensor cores or the FP64 pipe
+fdi_status launch_axis_f64(fdi_plan* p, const Field& f, int d, bool forward, const double* in, double* out,
+                           bool accumulate, const int* skip, cudaStream_t s);
 fdi_status launch_modes_f64(fdi_plan* p, const double* in, double* out, const double* T_all, int n, int nx,
                             int ny, const int* skip, cudaStream_t s);
 fdi_status launch_divide_modes_f64(fdi_plan* p, const Field& f, double sigma, double lambda, double* data,

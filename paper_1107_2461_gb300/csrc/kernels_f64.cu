@@ -1,9 +1,8 @@
 // FP64 kernels of the direct Helmholtz / Laplace inverse (the plain FP64 path).
 //
-//   k_lines_f64   out[l][k] = sum_j T[k][j] in[l][j]     transform along x (Eq. 25/29,
-//                 the factor E_x^{-1} or E_x applied to every x-line)
-//   k_slab_f64    out[b][k][c] = sum_j T[k][j] in[b][j][c]  transform along y per
-//                 z-slab, or along z over all columns (TPF)
+//   k_slab_f64    out[b][k][c] = sum_j T_b[k][j] in[b][j][c]  radial transforms of
+//                 the cylindrical TPF, one matrix per theta mode (the other
+//                 transforms: slice_transform.cu)
 //   k_thomas_f64  per (x-mode, y-mode) line the tridiagonal z-system
 //                 [(sigma - lam (Lx_i + Ly_j)) M_z - lam K_z] u = M_z f   (TPT,
 //                 end of Sec. 3: Thomas algorithm in one direction)
@@ -12,12 +11,13 @@
 //                 and per-block partial sums of r^2 and b^2 (fixed grid, so the
 //                 reduction order is deterministic)
 //
-// GB300 runs FP64 at about 2 FMA/clk/SM, so the transforms are FP64-pipe bound;
-// they are register-tiled (4x4 outputs per thread, 64x64 tiles staged in shared
+// GB300 runs FP64 at about 2 FMA/clk/SM, so k_slab_f64 is FP64-pipe bound; it is
+// register-tiled (4x4 outputs per thread, 64x64 tiles staged in shared
 // memory) so that every shared-memory load feeds two FMAs.
 #include <cmath>
 
 #include "fdi_internal.h"
+#include "slice_transform.h"
 
 namespace fdi {
 namespace {
@@ -26,61 +26,6 @@ constexpr int TB = 64;   // tile edge
 constexpr int TK = 16;   // k-chunk
 constexpr int kResBlocks = 152 * 8;
 constexpr int kResThreads = 256;
-
-template <bool ACC>
-__global__ void __launch_bounds__(256) k_lines_f64(const double* __restrict__ A, double* __restrict__ C,
-                                                   const double* __restrict__ T, int nin, int nout,
-                                                   long long L, const int* __restrict__ skip) {
-  if (skip && *skip) return;
-  __shared__ double As[TK][TB + 1];  // [j][line]
-  __shared__ double Bs[TK][TB + 1];  // [j][k]
-  const long long l0 = (long long)blockIdx.x * TB;
-  const int k0 = blockIdx.y * TB;
-  const int tx = threadIdx.x % 16, ty = threadIdx.x / 16;
-  double acc[4][4];
-#pragma unroll
-  for (int a = 0; a < 4; ++a)
-#pragma unroll
-    for (int b = 0; b < 4; ++b) acc[a][b] = 0.0;
-  for (int j0 = 0; j0 < nin; j0 += TK) {
-#pragma unroll
-    for (int r = 0; r < 4; ++r) {
-      int jj = threadIdx.x % TK, ll = threadIdx.x / TK + 16 * r;
-      long long line = l0 + ll;
-      int j = j0 + jj, k = k0 + ll;
-      As[jj][ll] = (line < L && j < nin) ? A[line * nin + j] : 0.0;
-      Bs[jj][ll] = (k < nout && j < nin) ? T[(long long)k * nin + j] : 0.0;
-    }
-    __syncthreads();
-#pragma unroll
-    for (int jj = 0; jj < TK; ++jj) {
-      double a[4], b[4];
-#pragma unroll
-      for (int q = 0; q < 4; ++q) {
-        a[q] = As[jj][ty + 16 * q];
-        b[q] = Bs[jj][tx + 16 * q];
-      }
-#pragma unroll
-      for (int q = 0; q < 4; ++q)
-#pragma unroll
-        for (int c = 0; c < 4; ++c) acc[q][c] = fma(a[q], b[c], acc[q][c]);
-    }
-    __syncthreads();
-  }
-#pragma unroll
-  for (int q = 0; q < 4; ++q) {
-    long long line = l0 + ty + 16 * q;
-    if (line >= L) continue;
-#pragma unroll
-    for (int c = 0; c < 4; ++c) {
-      int k = k0 + tx + 16 * c;
-      if (k < nout) {
-        long long idx = line * nout + k;
-        C[idx] = ACC ? C[idx] + acc[q][c] : acc[q][c];
-      }
-    }
-  }
-}
 
 // Element (j, c) of the input of batch b at A[b * zin + j * rs + c], of the
 // output C[b * zout + k * rs + c]; the matrix of batch b is T + b * tz (tz = 0:
@@ -521,26 +466,33 @@ StencilArgs stencil_args(const Field& f) {
 
 }  // namespace
 
-fdi_status launch_lines_f64(fdi_plan* p, const double* in, double* out, const double* T, int nin, int nout,
-                            long long lines, bool accumulate, const int* skip, cudaStream_t s) {
-  FDI_KTIMER(p, "transform_x_f64", s);
-  dim3 grid((unsigned)((lines + TB - 1) / TB), (unsigned)((nout + TB - 1) / TB));
-  if (accumulate)
-    k_lines_f64<true><<<grid, 256, 0, s>>>(in, out, T, nin, nout, lines, skip);
-  else
-    k_lines_f64<false><<<grid, 256, 0, s>>>(in, out, T, nin, nout, lines, skip);
-  FDI_LAUNCH_CHECK(p);
-  return FDI_OK;
-}
-
-fdi_status launch_slab_f64(fdi_plan* p, const double* in, double* out, const double* T, int nin, int nout,
-                           long long ncols, int batch, const int* skip, cudaStream_t s) {
-  FDI_KTIMER(p, batch > 1 ? "transform_y_f64" : "transform_z_f64", s);
-  dim3 grid((unsigned)((ncols + TB - 1) / TB), (unsigned)((nout + TB - 1) / TB), (unsigned)batch);
-  k_slab_f64<<<grid, 256, 0, s>>>(in, out, T, nin, nout, ncols, ncols, (long long)nin * ncols,
-                                  (long long)nout * ncols, 0LL, skip);
-  FDI_LAUNCH_CHECK(p);
-  return FDI_OK;
+fdi_status launch_axis_f64(fdi_plan* p, const Field& f, int d, bool forward, const double* in, double* out,
+                           bool accumulate, const int* skip, cudaStream_t s) {
+  const Axis* ax = f.ax[d];
+  const long long nx = f.n[0], ny = f.n[1];
+  FDI_KTIMER(p, d == 0 ? "transform_x_f64" : (d == 1 ? "transform_y_f64" : "transform_z_f64"), s);
+  const SliceAxis* sa = static_cast<const SliceAxis*>(ax->slices);
+  if (!sa) {
+    set_error("direction has no FP64 transform");
+    return FDI_ERR_INVALID_ARG;
+  }
+  SliceLines g;
+  g.R = f.P / ax->n;
+  if (d == 0) {  // x lines: rows (z, y)
+    g.S = g.R;
+    g.rs = nx;
+    g.ks = 1;
+  } else if (d == 1) {  // y lines: (z, x)
+    g.S = nx;
+    g.slab = nx * ny;
+    g.rs = 1;
+    g.ks = nx;
+  } else {  // z lines: (y, x)
+    g.S = nx * ny;
+    g.rs = 1;
+    g.ks = nx * ny;
+  }
+  return launch_slice_transform(p, forward ? sa->fwd : sa->bwd, in, out, g, accumulate, skip, s);
 }
 
 fdi_status launch_modes_f64(fdi_plan* p, const double* in, double* out, const double* T_all, int n, int nx,

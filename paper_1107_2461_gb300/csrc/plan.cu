@@ -12,6 +12,7 @@
 #include <utility>
 
 #include "fdi_internal.h"
+#include "slice_transform.h"
 
 namespace fdi {
 
@@ -177,6 +178,7 @@ fdi_status make_axis(Axis** out, const std::vector<double>& m, const std::vector
 void free_axis(Axis* ax) {
   if (!ax) return;
   mixed_free_axis(ax);
+  slice_free_axis(ax);
   void* ptrs[] = {ax->m, ax->kd, ax->ko, ax->wp, ax->wm, ax->w0, ax->lam, ax->E, ax->Einv};
   for (void* q : ptrs)
     if (q) cudaFree(q);
@@ -382,7 +384,17 @@ fdi_status finish_plan(fdi_plan* p, cudaStream_t s) {
   p->npartials = 16384;  // per-block partial sums of the reductions (>= blocks of any reduction grid)
   FDI_TRY(alloc_workspace(p));
   FDI_CUDA_TRY(cudaMallocHost((void**)&p->h_flag, sizeof(int) * 4));
-  if (p->prec != FDI_PREC_FP64) FDI_TRY(mixed_setup(p));
+  if (p->prec != FDI_PREC_FP64) {
+    FDI_TRY(mixed_setup(p));
+  } else {
+    // digit planes of the transformed directions (z only for the Cartesian TPF)
+    FDI_TRY(dev_alloc(&p->d_err, 1));
+    FDI_CUDA_TRY(cudaMemsetAsync(p->d_err, 0, sizeof(int), s));
+    const int nd = (p->thomas_axis == -1 && !p->cyl) ? 3 : 2;
+    for (int fi = 0; fi < p->nfields; ++fi)
+      for (int d = 0; d < nd; ++d) FDI_TRY(slice_prepare_axis(p, p->fields[fi].ax[d], s));
+    FDI_CUDA_TRY(cudaStreamSynchronize(s));
+  }
   if (p->grid == FDI_GRID_MAC) {
     FDI_TRY(stokes_setup(p));
     // three more workspaces and streams for the concurrent velocity solves

@@ -90,7 +90,8 @@ std::vector<double> tanh_faces(int n, double beta) {
 
 // Device bytes a MAC Stokes plan allocates (upper estimate of plan.cu,
 // mixed.cu, tc_transform.cu and stokes.cu): per direction and kind the FP64
-// operator and eigen data (+ split fp16 copies for mixed plans), four per-solve
+// operator and eigen data (+ split fp16 copies for mixed plans, digit planes
+// for FP64 ones), four per-solve
 // workspaces (five FP64 fields, partials, the mixed FP32 planes), and the
 // Krylov / face vectors.
 extern "C" size_t fdi_stokes_plan_bytes_estimate(const int n[3], int prec) {
@@ -98,7 +99,8 @@ extern "C" size_t fdi_stokes_plan_bytes_estimate(const int n[3], int prec) {
   size_t b = 0;
   for (int d = 0; d < 3; ++d) {
     const size_t nd = (size_t)n[d] + 1;
-    const size_t per_axis = 2 * nd * nd * 8 + 8 * nd * 8 + (prec != FDI_PREC_FP64 ? 2 * 2 * 2 * (nd + 32) * (nd + 32) * 2 : 0);
+    const size_t per_axis = 2 * nd * nd * 8 + 8 * nd * 8 + (prec != FDI_PREC_FP64 ? 2 * 2 * 2 * (nd + 32) * (nd + 32) * 2
+                                                     : 2 * (8 * 2 * (nd + 128) * (nd + 16) + 4 * (nd + 128)));
     b += 3 * per_axis;  // cell-Dirichlet, cell-Neumann, face kinds
   }
   const size_t Pp = (size_t)(n[0] + 4) * (n[1] + 4) * n[2];  // padded FP32 rows

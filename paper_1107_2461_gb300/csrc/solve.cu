@@ -63,29 +63,32 @@ fdi_status solve_once_f64(fdi_plan* p, int field, double sigma, double lambda, c
   double* t0 = p->ws[0];
   double* t1 = p->ws[1];
   double* t2 = p->ws[2];
-  const Axis* ax = f.ax[0];
-  const Axis* ay = f.ax[1];
-  const Axis* az = f.ax[2];
-  FDI_TRY(launch_lines_f64(p, in, t0, ax->Einv, nx, nx, (long long)ny * nz, false, skip, s));
-  FDI_TRY(launch_slab_f64(p, t0, t1, ay->Einv, ny, ny, nx, nz, skip, s));
+  auto fwd = [&](int d, const double* src, double* dst) {
+    return launch_axis_f64(p, f, d, true, src, dst, false, skip, s);
+  };
+  auto back = [&](int d, const double* src, double* dst, bool acc) {
+    return launch_axis_f64(p, f, d, false, src, dst, acc, skip, s);
+  };
+  FDI_TRY(fwd(0, in, t0));
+  FDI_TRY(fwd(1, t0, t1));
   if (p->thomas_axis == 2) {
     FDI_TRY(launch_thomas_f64(p, f, sigma, lambda, field, t1, t0, t2, skip, s));
-    FDI_TRY(launch_slab_f64(p, t0, t1, ay->E, ny, ny, nx, nz, skip, s));
-    FDI_TRY(launch_lines_f64(p, t1, out, ax->E, nx, nx, (long long)ny * nz, accumulate, skip, s));
+    FDI_TRY(back(1, t0, t1, false));
+    FDI_TRY(back(0, t1, out, accumulate));
   } else if (p->cyl) {
     // cylindrical TPF (Eq. 45-46): the radial transform of theta mode j uses
     // that mode's own eigenbasis, the divide its own eigenvalues
     FDI_TRY(launch_modes_f64(p, t1, t0, p->cyl_Eri, nz, nx, ny, skip, s));
     FDI_TRY(launch_divide_modes_f64(p, f, sigma, lambda, t0, skip, s));
     FDI_TRY(launch_modes_f64(p, t0, t1, p->cyl_Er, nz, nx, ny, skip, s));
-    FDI_TRY(launch_slab_f64(p, t1, t0, ay->E, ny, ny, nx, nz, skip, s));
-    FDI_TRY(launch_lines_f64(p, t0, out, ax->E, nx, nx, (long long)ny * nz, accumulate, skip, s));
+    FDI_TRY(back(1, t1, t0, false));
+    FDI_TRY(back(0, t0, out, accumulate));
   } else {
-    FDI_TRY(launch_slab_f64(p, t1, t0, az->Einv, nz, nz, (long long)nx * ny, 1, skip, s));
+    FDI_TRY(fwd(2, t1, t0));
     FDI_TRY(launch_divide_f64(p, f, sigma, lambda, t0, skip, s));
-    FDI_TRY(launch_slab_f64(p, t0, t1, az->E, nz, nz, (long long)nx * ny, 1, skip, s));
-    FDI_TRY(launch_slab_f64(p, t1, t0, ay->E, ny, ny, nx, nz, skip, s));
-    FDI_TRY(launch_lines_f64(p, t0, out, ax->E, nx, nx, (long long)ny * nz, accumulate, skip, s));
+    FDI_TRY(back(2, t0, t1, false));
+    FDI_TRY(back(1, t1, t0, false));
+    FDI_TRY(back(0, t0, out, accumulate));
   }
   return FDI_OK;
 }
