@@ -130,11 +130,30 @@ __global__ void k_finalize_out(const float* __restrict__ xh, const float* __rest
   }
 }
 
+// end of a first-pass block (8 warps): the components' sums, one lane each, and
+// one atomic for max |b|
+__device__ __forceinline__ void init_block_out(const ResidArgs& a, const double* sh, const float* smax, int nc) {
+  if (threadIdx.x >= 32) return;
+  const int lane = threadIdx.x;
+  if (lane < 4) {
+    double t = 0.0;
+    if (lane > 0 && lane < nc)
+      for (int q = 0; q < 8; ++q) t += sh[4 * q + lane];
+    a.partials[4 * blockIdx.x + lane] = t;
+  }
+  float m = lane < 8 ? smax[lane] : 0.f;
+#pragma unroll
+  for (int o = 4; o > 0; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
+  if (lane == 0 && m > 0.f) atomicMax(reinterpret_cast<unsigned int*>(a.rmax), __float_as_uint(m));
+  __syncwarp();  // the record is written before thread 0 fences and takes the ticket
+}
+
 // r_0 = b: FP64 -> FP32 copy into the padded residual layout, ||b||^2, max |b|
 // and (singular problems) the volume-weighted sums; one warp per x-line
 __global__ void __launch_bounds__(256) k_init_rhs(ResidArgs a) {
   pdl_wait();
   __shared__ double sh[4 * 8];
+  __shared__ float smax[8];
   const int nx = a.nx, ny = a.ny, nz = a.nz;
   const int warp = threadIdx.x / 32, lane = threadIdx.x % 32;
   const int nwarps = gridDim.x * 8;
@@ -171,24 +190,26 @@ __global__ void __launch_bounds__(256) k_init_rhs(ResidArgs a) {
       }
     }
   }
-  double w[4] = {0.0, (double)sbb, df::to_f64(svb), df::to_f64(sv)};
+  // within the warp in double-float (the FP64 pipe adds 2 lanes per clock)
+  df::F2 sb = df::make(sbb, 0.f);
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) {
-#pragma unroll
-    for (int q = 0; q < 4; ++q) w[q] += __shfl_down_sync(0xffffffffu, w[q], o);
+    sb = df::add(sb, df::make(__shfl_xor_sync(0xffffffffu, sb.hi, o), __shfl_xor_sync(0xffffffffu, sb.lo, o)));
     rmax = fmaxf(rmax, __shfl_xor_sync(0xffffffffu, rmax, o));
+    if (a.want_mean) {
+      svb = df::add(svb, df::make(__shfl_xor_sync(0xffffffffu, svb.hi, o), __shfl_xor_sync(0xffffffffu, svb.lo, o)));
+      sv = df::add(sv, df::make(__shfl_xor_sync(0xffffffffu, sv.hi, o), __shfl_xor_sync(0xffffffffu, sv.lo, o)));
+    }
   }
   if (lane == 0) {
-    for (int q = 0; q < 4; ++q) sh[4 * warp + q] = w[q];
-    if (rmax > 0.f) atomicMax(reinterpret_cast<unsigned int*>(a.rmax), __float_as_uint(rmax));
+    sh[4 * warp] = 0.0;
+    sh[4 * warp + 1] = df::to_f64(sb);
+    sh[4 * warp + 2] = df::to_f64(svb);
+    sh[4 * warp + 3] = df::to_f64(sv);
+    smax[warp] = rmax;
   }
   __syncthreads();
-  if (threadIdx.x == 0) {
-    double t[4] = {0, 0, 0, 0};
-    for (int q = 0; q < 8; ++q)
-      for (int c = 0; c < 4; ++c) t[c] += sh[4 * q + c];
-    for (int c = 0; c < 4; ++c) a.partials[4 * blockIdx.x + c] = t[c];
-  }
+  init_block_out(a, sh, smax, a.want_mean ? 4 : 2);
   finish_if_last(a.fin, threadIdx.x, blockDim.x);
 }
 
@@ -197,7 +218,8 @@ __global__ void __launch_bounds__(256) k_init_rhs(ResidArgs a) {
 // ||b||^2 and max |b|
 __global__ void __launch_bounds__(256) k_init_rhs_flat(ResidArgs a, long long P) {
   pdl_wait();
-  __shared__ double sh[8];
+  __shared__ double sh[4 * 8];
+  __shared__ float smax[8];
   const int warp = threadIdx.x / 32, lane = threadIdx.x % 32;
   float sbb = 0.f, rmax = 0.f;
   const long long stride = (long long)gridDim.x * blockDim.x * 8;
@@ -237,18 +259,11 @@ __global__ void __launch_bounds__(256) k_init_rhs_flat(ResidArgs a, long long P)
     rmax = fmaxf(rmax, __shfl_xor_sync(0xffffffffu, rmax, o));
   }
   if (lane == 0) {
-    sh[warp] = (double)sbb;
-    if (rmax > 0.f) atomicMax(reinterpret_cast<unsigned int*>(a.rmax), __float_as_uint(rmax));
+    sh[4 * warp + 1] = (double)sbb;
+    smax[warp] = rmax;
   }
   __syncthreads();
-  if (threadIdx.x == 0) {
-    double t = 0.0;
-    for (int q = 0; q < 8; ++q) t += sh[q];
-    a.partials[4 * blockIdx.x + 0] = 0.0;
-    a.partials[4 * blockIdx.x + 1] = t;
-    a.partials[4 * blockIdx.x + 2] = 0.0;
-    a.partials[4 * blockIdx.x + 3] = 0.0;
-  }
+  init_block_out(a, sh, smax, 2);
   finish_if_last(a.fin, threadIdx.x, blockDim.x);
 }
 
@@ -1195,8 +1210,11 @@ fdi_status mixed_field_solve(fdi_plan* p, int field, double sigma, double lambda
   ra.st = p->d_status;
   ra.partials = p->partials;
 
-  // r_0 = b (and the volume-weighted mean of b for the singular problem)
-  const int iblocks = 152 * 8;
+  // r_0 = b (and the volume-weighted mean of b for the singular problem); the
+  // flat form needs no more blocks than it has groups of 8 values per thread
+  // (each block costs a partial record and a ticket; with the packed sums a
+  // 64^3 first pass went from 21 to 15 us between events)
+  const int iblocks = 152 * 8, fblocks = (int)std::min<long long>(iblocks, (f.P + 2047) / 2048);
   {
     FDI_KTIMER(p, "residual_df_init", s);
     ResidArgs a0 = ra;
@@ -1208,7 +1226,7 @@ fdi_status mixed_field_solve(fdi_plan* p, int field, double sigma, double lambda
     a0.rmax = p->d_scales + 0;
     a0.fin = FinishArgs{p->d_counter, p->partials, p->d_status, p->tol, 0, singular ? 1 : 0};
     if (px == nx && !singular && (reinterpret_cast<uintptr_t>(b) & 15u) == 0)
-      FDI_CUDA_TRY(launch_pdl(true, k_init_rhs_flat, dim3(iblocks), dim3(256), 0, s, a0, f.P));
+      FDI_CUDA_TRY(launch_pdl(true, k_init_rhs_flat, dim3(fblocks), dim3(256), 0, s, a0, f.P));
     else  // one warp per x-line: no more blocks than lines / 8
       FDI_CUDA_TRY(launch_pdl(true, k_init_rhs, dim3(std::min(iblocks, (ny * nz + 7) / 8)), dim3(256), 0, s, a0));
     FDI_LAUNCH_CHECK(p);

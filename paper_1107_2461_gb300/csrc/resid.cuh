@@ -7,6 +7,7 @@
 
 #include "df.cuh"
 #include "fdi_internal.h"
+#include "reduce.cuh"
 
 namespace fdi {
 namespace {
@@ -236,6 +237,7 @@ __device__ __forceinline__ void resid_body(const ResidArgs& a, double* sh, int b
     Va = df::mul(ld2(a.m[0] + ia), my);
     Vb = df::mul(ld2(a.m[0] + ib), my);
   }
+  __shared__ float smax[kResTY];
   float srr = 0.f, sbb = 0.f, rmax = 0.f;
   df::F2 svb = df::make(0.f, 0.f), sv = df::make(0.f, 0.f);
   // Per-row base pointers and 32-bit plane offsets (every field has fewer
@@ -505,14 +507,22 @@ __device__ __forceinline__ void resid_body(const ResidArgs& a, double* sh, int b
     sh[4 * wy + 1] = (double)sbb;
     sh[4 * wy + 2] = MEAN ? df::to_f64(svb) : 0.0;
     sh[4 * wy + 3] = MEAN ? df::to_f64(sv) : 0.0;
-    if (rmax > 0.f) atomicMax(reinterpret_cast<unsigned int*>(a.rmax), __float_as_uint(rmax));
+    smax[wy] = rmax;
   }
   __syncthreads();
-  if (lane == 0 && wy == 0) {
-    double t[4] = {0, 0, 0, 0};
-    for (int q = 0; q < kResTY; ++q)
-      for (int c = 0; c < 4; ++c) t[c] += sh[4 * q + c];
-    for (int c = 0; c < 4; ++c) a.partials[4 * bid + c] = t[c];
+  if (wy == 0) {
+    // one lane per component (a chain of FP64 adds each), one atomic per block
+    if (lane < 4) {
+      double t = 0.0;
+      if (MEAN || lane < (MODE == 0 ? 2 : 1))
+        for (int q = 0; q < kResTY; ++q) t += sh[4 * q + lane];
+      a.partials[4 * bid + lane] = t;
+    }
+    float m = lane < kResTY ? smax[lane] : 0.f;
+#pragma unroll
+    for (int o = kResTY / 2; o > 0; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
+    if (lane == 0 && m > 0.f) atomicMax(reinterpret_cast<unsigned int*>(a.rmax), __float_as_uint(m));
+    __syncwarp();  // the record is written before thread 0 fences and takes the ticket
   }
 }
 
@@ -540,38 +550,51 @@ __device__ void finish_block(const double* __restrict__ partials, int nblocks, D
                              int want_mean, int t, int nt) {
   __shared__ double shf[4 * 32];
   double s[4] = {0, 0, 0, 0};
-  // 8 partial records per thread in flight (16-byte loads), fixed order
+  // 8 partial records per thread in flight (16-byte loads), fixed order; a
+  // first check without the mean reads components 0 and 1 only, a later one 0
   const double2* p2 = reinterpret_cast<const double2*>(partials);
   for (int q0 = t; q0 < nblocks; q0 += 8 * nt) {
     double2 v[8][2];
 #pragma unroll
     for (int u = 0; u < 8; ++u) {
       const int q = q0 + u * nt;
+      v[u][0] = v[u][1] = make_double2(0.0, 0.0);
       if (q < nblocks) {
         v[u][0] = p2[2 * q];
-        v[u][1] = p2[2 * q + 1];
-      } else {
-        v[u][0] = v[u][1] = make_double2(0.0, 0.0);
+        if (want_mean) v[u][1] = p2[2 * q + 1];
       }
     }
 #pragma unroll
     for (int u = 0; u < 8; ++u) {
+      if (q0 - (t & 31) + u * nt >= nblocks) break;  // nothing for this warp
       s[0] += v[u][0].x;
       s[1] += v[u][0].y;
-      s[2] += v[u][1].x;
-      s[3] += v[u][1].y;
+      if (want_mean) {
+        s[2] += v[u][1].x;
+        s[3] += v[u][1].y;
+      }
     }
   }
-  for (int o = 16; o > 0; o >>= 1)
-    for (int c = 0; c < 4; ++c) s[c] += __shfl_down_sync(0xffffffffu, s[c], o);
-  const int w = t / 32, ln = t % 32;
-  if (ln == 0)
-    for (int c = 0; c < 4; ++c) shf[4 * w + c] = s[c];
+  // only the warps that hold records take part
+  const int w = t / 32, ln = t % 32, nw = min(nt / 32, (nblocks + 31) / 32);
+  if (w < nw) {
+    // lanes 0, 16, 8, 24: components 0, 1, 2, 3
+    const double v = want_mean ? red::warp_sum4(s[0], s[1], s[2], s[3]) : red::warp_sum2(s[0], s[1]);
+    if (ln == 0) shf[4 * w] = v;
+    if (ln == 16) shf[4 * w + 1] = v;
+    if (want_mean && ln == 8) shf[4 * w + 2] = v;
+    if (want_mean && ln == 24) shf[4 * w + 3] = v;
+  }
   __syncthreads();
+  if (w != 0) return;
+  // one lane per component over the warps
+  double c = 0.0;
+  if (ln < (want_mean ? 4 : 2))
+    for (int q = 0; q < nw; ++q) c += shf[4 * q + ln];
+  double tt[4];
+#pragma unroll
+  for (int q = 0; q < 4; ++q) tt[q] = __shfl_sync(0xffffffffu, c, q);
   if (t != 0) return;
-  double tt[4] = {0, 0, 0, 0};
-  for (int q = 0; q < nt / 32; ++q)
-    for (int c = 0; c < 4; ++c) tt[c] += shf[4 * q + c];
   if (kind == 0) {
     // the solve's status starts here (no kernel of the solve reads it before)
     st->tol_used = tol;

@@ -31,6 +31,7 @@
 #include <vector>
 
 #include "fdi_internal.h"
+#include "reduce.cuh"
 #include "resident.h"
 
 namespace fdi {
@@ -50,6 +51,9 @@ namespace {
 
 constexpr int kDotBlocks = 152 * 4;
 constexpr int kDotThreads = 256;
+// blocks of a reduction over n values: at least 1024 values (4 per thread) each,
+// since every block costs a partial record and a ticket
+int dot_blocks(long long n) { return (int)std::max<long long>(1, std::min<long long>(kDotBlocks, n / 1024)); }
 
 struct MacGeom {
   int nx, ny, nz;
@@ -108,27 +112,9 @@ __global__ void k_div(MacGeom g, const double* __restrict__ hu, const double* __
   y[((long long)k * ny + j) * nx + i] = (ur - ul) * g.ih[0][i] + (vr - vl) * g.ih[1][j] + (wr - wl) * g.ih[2][k];
 }
 
-__device__ __forceinline__ void block_reduce2(double& a, double& b) {
-  __shared__ double sh[2 * (kDotThreads / 32)];
-  for (int o = 16; o > 0; o >>= 1) {
-    a += __shfl_down_sync(0xffffffffu, a, o);
-    b += __shfl_down_sync(0xffffffffu, b, o);
-  }
-  const int w = threadIdx.x / 32, ln = threadIdx.x % 32;
-  if (ln == 0) {
-    sh[2 * w] = a;
-    sh[2 * w + 1] = b;
-  }
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    double sa = 0, sb = 0;
-    for (int q = 0; q < kDotThreads / 32; ++q) {
-      sa += sh[2 * q];
-      sb += sh[2 * q + 1];
-    }
-    a = sa;
-    b = sb;
-  }
+__device__ __forceinline__ void block_reduce2(double& a, double& b, int warps = kDotThreads / 32) {
+  __shared__ double sh[32];
+  red::block_sum2(a, b, warps, sh);
 }
 
 __device__ void kry_finish_last(const double* partials, KryState* st, int kind, unsigned* ticket);
@@ -151,13 +137,17 @@ __global__ void __launch_bounds__(kDotThreads) k_dot2(const double* __restrict__
 }
 
 __device__ __forceinline__ void sum_partials(const double* partials, double& a, double& b) {
+  const int nb = (int)gridDim.x;
+  const double2* p2 = reinterpret_cast<const double2*>(partials);
   a = 0.0;
   b = 0.0;
-  for (int q = threadIdx.x; q < kDotBlocks; q += blockDim.x) {
-    a += partials[2 * q];
-    b += partials[2 * q + 1];
+  for (int q = threadIdx.x; q < nb; q += blockDim.x) {
+    const double2 v = p2[q];
+    a += v.x;
+    b += v.y;
   }
-  block_reduce2(a, b);
+  __syncthreads();  // the block's own sums are done with the shared array
+  block_reduce2(a, b, min(kDotThreads / 32, (nb + 31) / 32));
 }
 
 // kinds of scalar updates after a reduction (KF_L2_*: BiCGstab(2))
@@ -752,7 +742,7 @@ fdi_status cmatvec(fdi_plan* p, const MacGeom& g, double lambda, double* q, doub
 fdi_status wdots(fdi_plan* p, const MacGeom& g, const double* a, const double* b, const double* c, int kind,
                  cudaStream_t s) {
   FDI_KTIMER(p, "stokes_dot", s);
-  k_wdot<<<kDotBlocks, kDotThreads, 0, s>>>(g, a, b, c, p->kpartials, p->d_kry, kind, p->kticket);
+  k_wdot<<<dot_blocks(p->fields[FDI_FIELD_CELL].P), kDotThreads, 0, s>>>(g, a, b, c, p->kpartials, p->d_kry, kind, p->kticket);
   FDI_LAUNCH_CHECK(p);
   return FDI_OK;
 }
@@ -760,7 +750,7 @@ fdi_status wdots(fdi_plan* p, const MacGeom& g, const double* a, const double* b
 fdi_status dots(fdi_plan* p, const double* a, const double* b, const double* c, const double* d, long long n,
                 int kind, cudaStream_t s) {
   FDI_KTIMER(p, "stokes_dot", s);
-  k_dot2<<<kDotBlocks, kDotThreads, 0, s>>>(a, b, c, d, n, p->kpartials, p->d_kry, kind, p->kticket);
+  k_dot2<<<dot_blocks(n), kDotThreads, 0, s>>>(a, b, c, d, n, p->kpartials, p->d_kry, kind, p->kticket);
   FDI_LAUNCH_CHECK(p);
   return FDI_OK;
 }
@@ -938,7 +928,7 @@ fdi_status stokes_solve(fdi_plan* p, double dt, double Re, const double* const f
       FDI_TRY(wdots(p, g, pv, v, nullptr, KF_CG_ALPHA, s));
       {
         FDI_KTIMER(p, "stokes_update", s);
-        k_cg_xr<<<kDotBlocks, kDotThreads, 0, s>>>(p->d_kry, x, r, pv, v, Pc, p->kpartials, p->d_kry, KF_CG_ITER,
+        k_cg_xr<<<dot_blocks(Pc), kDotThreads, 0, s>>>(p->d_kry, x, r, pv, v, Pc, p->kpartials, p->d_kry, KF_CG_ITER,
                                                    p->kticket);
         FDI_LAUNCH_CHECK(p);
       }
@@ -986,7 +976,7 @@ fdi_status stokes_solve(fdi_plan* p, double dt, double Re, const double* const f
       FDI_TRY(dots(p, r2, r2, r0, r2, Pc, KF_L2_MR2, s));
       {
         FDI_KTIMER(p, "stokes_update", s);
-        k_l2_final<<<kDotBlocks, kDotThreads, 0, s>>>(p->d_kry, x, r0, r1, r2, u0, u1, u2, Pc, p->kpartials,
+        k_l2_final<<<dot_blocks(Pc), kDotThreads, 0, s>>>(p->d_kry, x, r0, r1, r2, u0, u1, u2, Pc, p->kpartials,
                                                       p->d_kry, KF_L2_CONV, p->kticket);
         FDI_LAUNCH_CHECK(p);
       }
@@ -1013,7 +1003,7 @@ fdi_status stokes_solve(fdi_plan* p, double dt, double Re, const double* const f
       FDI_TRY(dots(p, t, sv, t, t, Pc, KF_OMEGA, s));
       {
         FDI_KTIMER(p, "stokes_update", s);
-        k_bicg_xr<<<kDotBlocks, kDotThreads, 0, s>>>(p->d_kry, x, y, z, r, sv, t, rhat, Pc, p->kpartials, p->d_kry,
+        k_bicg_xr<<<dot_blocks(Pc), kDotThreads, 0, s>>>(p->d_kry, x, y, z, r, sv, t, rhat, Pc, p->kpartials, p->d_kry,
                                                      KF_ITER, p->kticket);
         FDI_LAUNCH_CHECK(p);
       }
@@ -1023,7 +1013,7 @@ fdi_status stokes_solve(fdi_plan* p, double dt, double Re, const double* const f
   }
   // zero-mean pressure q -> p = q / dt
   {
-    k_vsum<<<kDotBlocks, kDotThreads, 0, s>>>(g, x, p->kpartials, p->d_kry + 1, KF_MEAN, p->kticket);
+    k_vsum<<<dot_blocks(Pc), kDotThreads, 0, s>>>(g, x, p->kpartials, p->d_kry + 1, KF_MEAN, p->kticket);
     FDI_LAUNCH_CHECK(p);
     k_pressure<<<vb, vt, 0, s>>>(p->d_kry + 1, x, 1.0 / dt, pr, Pc);
     FDI_LAUNCH_CHECK(p);
