@@ -163,7 +163,8 @@ struct fdi_plan {
   // captured on its second occurrence and replayed with a single graph launch
   // afterwards (a small LRU set, so alternating buffers keep their graphs)
   bool use_graphs = true;
-  bool pdl = true;                  // programmatic dependent launch between the mixed solve's kernels
+  bool pdl = true;                  // programmatic dependent launch between a solve's kernels
+  bool loop_capture = false;        // capturing the body of the device-side Krylov loop
   // mixed field solves run one direct solve only (no residual check, no
   // refinement; FP64 output of the first solve): set around preconditioner
   // applications, which need no more than an approximate inverse
@@ -277,6 +278,12 @@ cudaError_t launch_pdl(bool pdl, void (*kernel)(KArgs...), dim3 grid, dim3 block
   return cudaLaunchKernelEx(&cfg, kernel, std::forward<Args>(args)...);
 }
 
+// the graph a stream is being captured into (null: not capturing)
+cudaGraph_t capturing_graph(cudaStream_t s);
+// add an IF node after the capture point of s (capturing into g); *body is its
+// body graph
+fdi_status graph_add_if(cudaStream_t s, cudaGraph_t g, cudaGraphConditionalHandle h, cudaGraph_t* body);
+
 // drop the captured solve graph (arguments or controls changed)
 void invalidate_graph(fdi_plan* p);
 
@@ -321,8 +328,10 @@ fdi_status eigen_decompose_batch(int count, int n, const double* m, const double
 // FP64 path launchers (kernels_f64.cu).  Transform of direction d of a field by
 // E_d^{-1} (forward) or E_d: out (+)= T in along every line of d (x lines may
 // accumulate), on the tensor cores or the FP64 pipe
+// (pdl: programmatic launch; not for the first kernel after a graph's
+// conditional node, a join or a copy)
 fdi_status launch_axis_f64(fdi_plan* p, const Field& f, int d, bool forward, const double* in, double* out,
-                           bool accumulate, const int* skip, cudaStream_t s);
+                           bool accumulate, bool pdl, const int* skip, cudaStream_t s);
 fdi_status launch_modes_f64(fdi_plan* p, const double* in, double* out, const double* T_all, int n, int nx,
                             int ny, const int* skip, cudaStream_t s);
 fdi_status launch_divide_modes_f64(fdi_plan* p, const Field& f, double sigma, double lambda, double* data,
@@ -338,13 +347,12 @@ fdi_status launch_thomas_f64(fdi_plan* p, const Field& f, double sigma, double l
                              double* out, double* scratch, const int* skip, cudaStream_t s);
 fdi_status launch_divide_f64(fdi_plan* p, const Field& f, double sigma, double lambda, double* data,
                              const int* skip, cudaStream_t s);
+// r = b - A u, its norm and the convergence check (first: the solve's status
+// starts here; next_round: captured graph's condition of the next round, or 0)
 fdi_status launch_residual_f64(fdi_plan* p, const Field& f, double sigma, double lambda, const double* b,
-                               const double* u, double* r, bool subtract_mean, const int* skip,
-                               cudaStream_t s);
-fdi_status launch_finish_residual(fdi_plan* p, int nblocks, bool first, int count_step, const int* skip,
-                                  cudaStream_t s);
+                               const double* u, double* r, bool subtract_mean, bool first,
+                               cudaGraphConditionalHandle next_round, const int* skip, cudaStream_t s);
 fdi_status launch_mean_f64(fdi_plan* p, const Field& f, const double* b, cudaStream_t s);
-fdi_status launch_reset_status(fdi_plan* p, cudaStream_t s);
 
 // solve orchestration (solve.cu)
 fdi_status field_solve(fdi_plan* p, int field, double sigma, double lambda, const double* rhs, double* out,

@@ -973,8 +973,6 @@ fdi_status mixed_alloc_workspace(fdi_plan* p) {
   p->wr1_plane = (long long)szr;
   FDI_CUDA_TRY(cudaMalloc(&p->d_scales, (size_t)(kMaxRefineCap + 2) * kScaleStride * sizeof(float)));
   FDI_CUDA_TRY(cudaMalloc(&p->lam_w, (size_t)10 * kMaxN * sizeof(float2)));
-  FDI_CUDA_TRY(cudaMalloc(&p->d_counter, 4 * sizeof(unsigned)));
-  FDI_CUDA_TRY(cudaMemset(p->d_counter, 0, 4 * sizeof(unsigned)));
   return FDI_OK;
 }
 
@@ -1430,45 +1428,23 @@ fdi_status mixed_field_solve(fdi_plan* p, int field, double sigma, double lambda
   // In a captured solve, round r >= 2 sits in a conditional graph node placed
   // (nested) in round r-1's graph, whose residual check sets the condition, so
   // a converged solve launches nothing more.
-  cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
-  cudaGraph_t cgraph = nullptr;
   bool conditional = false;
-  if (!one_pass && p->max_refine >= 2 && p->cstream &&
-      cudaStreamGetCaptureInfo(s, &cap, nullptr, &cgraph, nullptr, nullptr, nullptr) == cudaSuccess &&
-      cap == cudaStreamCaptureStatusActive && cgraph) {
-    // add an IF node after the current capture point of `st` (capturing into
-    // `g`); returns its body graph
-    auto add_if = [&](cudaStream_t st, cudaGraph_t g, cudaGraphConditionalHandle h, cudaGraph_t* body) -> fdi_status {
-      const cudaGraphNode_t* deps = nullptr;
-      size_t ndeps = 0;
-      cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
-      cudaGraph_t gg = nullptr;
-      FDI_CUDA_TRY(cudaStreamGetCaptureInfo(st, &cs, nullptr, &gg, &deps, nullptr, &ndeps));
-      cudaGraphNodeParams cp = {};
-      cp.type = cudaGraphNodeTypeConditional;
-      cp.conditional.handle = h;
-      cp.conditional.type = cudaGraphCondTypeIf;
-      cp.conditional.size = 1;
-      cudaGraphNode_t node = nullptr;
-      FDI_CUDA_TRY(cudaGraphAddNode(&node, g, deps, nullptr, ndeps, &cp));
-      FDI_CUDA_TRY(cudaStreamUpdateCaptureDependencies(st, &node, nullptr, 1, cudaStreamSetCaptureDependencies));
-      *body = cp.conditional.phGraph_out[0];
-      return FDI_OK;
-    };
+  cudaGraph_t cgraph = (!one_pass && p->max_refine >= 2 && p->cstream) ? capturing_graph(s) : nullptr;
+  if (cgraph) {
     conditional = true;
     cudaGraphConditionalHandle h = 0;
     FDI_CUDA_TRY(cudaGraphConditionalHandleCreate(&h, cgraph, 0, cudaGraphCondAssignDefault));
     FDI_TRY(enqueue_round(0, s, 0));
     FDI_TRY(enqueue_round(1, s, h));
     cudaGraph_t body = nullptr;
-    FDI_TRY(add_if(s, cgraph, h, &body));
+    FDI_TRY(graph_add_if(s, cgraph, h, &body));
     for (int r = 2; r <= p->max_refine; ++r) {
       cudaGraphConditionalHandle hn = 0;
       if (r < p->max_refine) FDI_CUDA_TRY(cudaGraphConditionalHandleCreate(&hn, body, 0, cudaGraphCondAssignDefault));
       FDI_CUDA_TRY(cudaStreamBeginCaptureToGraph(p->cstream, body, nullptr, nullptr, 0, cudaStreamCaptureModeRelaxed));
       fdi_status st = enqueue_round(r, p->cstream, hn);
       cudaGraph_t next_body = nullptr;
-      if (st == FDI_OK && hn) st = add_if(p->cstream, body, hn, &next_body);
+      if (st == FDI_OK && hn) st = graph_add_if(p->cstream, body, hn, &next_body);
       cudaGraph_t done_graph = nullptr;
       const cudaError_t e = cudaStreamEndCapture(p->cstream, &done_graph);
       FDI_TRY(st);

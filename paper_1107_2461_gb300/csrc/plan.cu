@@ -220,6 +220,8 @@ fdi_status alloc_workspace(fdi_plan* p) {
   FDI_TRY(dev_alloc(&p->partials, (size_t)p->npartials * 4));
   FDI_TRY(dev_alloc(&p->d_status, 1));
   FDI_CUDA_TRY(cudaMemset(p->d_status, 0, sizeof(DevStatus)));
+  FDI_TRY(dev_alloc(&p->d_counter, 4));
+  FDI_CUDA_TRY(cudaMemset(p->d_counter, 0, 4 * sizeof(unsigned)));
   // FP64 TPT sweeps keep their line factors for repeated (sigma, lambda)
   if (p->prec == FDI_PREC_FP64 && p->thomas_axis == 2) FDI_TRY(alloc_thomas_cache(p, p->Pmax));
   return FDI_OK;
@@ -394,6 +396,7 @@ fdi_status finish_plan(fdi_plan* p, cudaStream_t s) {
     for (int fi = 0; fi < p->nfields; ++fi)
       for (int d = 0; d < nd; ++d) FDI_TRY(slice_prepare_axis(p, p->fields[fi].ax[d], s));
     FDI_CUDA_TRY(cudaStreamSynchronize(s));
+    FDI_CUDA_TRY(cudaStreamCreateWithFlags(&p->cstream, cudaStreamNonBlocking));
   }
   if (p->grid == FDI_GRID_MAC) {
     FDI_TRY(stokes_setup(p));

@@ -709,7 +709,8 @@ void slice_free_axis(Axis* ax) {
 }
 
 fdi_status launch_slice_transform(fdi_plan* p, const SliceMatrix& m, const double* in, double* out,
-                                  const SliceLines& g, bool accumulate, const int* skip, cudaStream_t s) {
+                                  const SliceLines& g, bool accumulate, bool pdl, const int* skip,
+                                  cudaStream_t s) {
   SliceArgs a{};
   a.in = in;
   a.out = out;
@@ -733,7 +734,7 @@ fdi_status launch_slice_transform(fdi_plan* p, const SliceMatrix& m, const doubl
   const int tn = wide ? 64 : 32;
   a.n_items = (int)((g.R + tn - 1) / tn) * m.m_tiles;
   const int grid = a.n_items < sms ? a.n_items : sms;
-  FDI_CUDA_TRY(launch_pdl(true, wide ? k_slice_transform<64> : k_slice_transform<32>, dim3((unsigned)grid),
+  FDI_CUDA_TRY(launch_pdl(pdl && p->pdl, wide ? k_slice_transform<64> : k_slice_transform<32>, dim3((unsigned)grid),
                           dim3(THREADS), (size_t)(wide ? Smem<64>::BYTES : Smem<32>::BYTES), s, a));
   FDI_LAUNCH_CHECK(p);
   return FDI_OK;

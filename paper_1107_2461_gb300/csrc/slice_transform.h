@@ -31,6 +31,7 @@ fdi_status slice_prepare_axis(fdi_plan* p, Axis* ax, cudaStream_t s);
 void slice_free_axis(Axis* ax);
 // out (+)= T in along every line; in and out distinct
 fdi_status launch_slice_transform(fdi_plan* p, const SliceMatrix& m, const double* in, double* out,
-                                  const SliceLines& g, bool accumulate, const int* skip, cudaStream_t s);
+                                  const SliceLines& g, bool accumulate, bool pdl, const int* skip,
+                                  cudaStream_t s);
 
 }  // namespace fdi

@@ -72,3 +72,41 @@ def test_power_of_two_scaling_is_exact(fdi, k):
     finally:
         plan.destroy()
     assert np.array_equal(np.ldexp(a, k), b)
+
+
+@pytest.mark.parametrize("n", [(31, 7, 2), (32, 8, 8), (33, 9, 9), (64, 8, 17), (65, 16, 3), (97, 17, 5), (2, 2, 33)])
+@pytest.mark.parametrize("walls", [(0, 0), (1, 1), (0, 1), (1, 0)])
+def test_residual_confirms_the_first_solve(fdi, n, walls):
+    # columns, rows and planes at the edges of the residual's blocks: a face or
+    # a wall missed there would leave a residual of order one, so the first check
+    # of a direct solve confirms it at the FP64 tolerance with no correction
+    import torch
+    plan = fdi.plan_create([tanh_faces(n[d], 1.5) for d in range(3)], n, (walls[0],) * 3, (walls[1],) * 3)
+    try:
+        for lam in (0.7, 0.0) if walls != (1, 1) else (0.7,):
+            f = torch.from_numpy(rhs_uniform(n[::-1], 3)).cuda()
+            out = torch.empty_like(f)
+            if lam:
+                fdi.helmholtz_solve(plan, lam, f, out)
+            else:
+                fdi.laplace_solve(plan, f, out)
+            torch.cuda.synchronize()
+            _, steps, rel, status = fdi.last_result(plan)
+            assert status == 0 and steps == 0 and rel <= 1e-11
+    finally:
+        plan.destroy()
+
+
+@pytest.mark.parametrize("n", [(31, 3, 33), (64, 9, 8), (5, 33, 70)])  # r, theta, z
+def test_residual_confirms_the_first_cylindrical_solve(fdi, n):
+    import torch
+    plan = fdi.plan_create_cyl(0.5 + tanh_faces(n[0], 1.0), n[1], tanh_faces(n[2], 1.0))
+    f = torch.from_numpy(rhs_uniform(n[::-1], 3)).cuda()
+    out = torch.empty_like(f)
+    try:
+        fdi.helmholtz_solve(plan, 0.3, f, out)
+        torch.cuda.synchronize()
+        _, steps, rel, status = fdi.last_result(plan)
+    finally:
+        plan.destroy()
+    assert status == 0 and steps == 0 and rel <= 1e-11
