@@ -337,8 +337,9 @@ fdi_status fdi_plan_autotune(fdi_plan* plan, double lambda, const double* rhs, d
  * field solve whose arguments (field, sigma, lambda, rhs, out, stream) repeat
  * those of the previous call on this plan is captured into a CUDA graph on its
  * second occurrence and replayed as one graph launch from then on; results are
- * identical to the eager launch sequence.  The legacy default stream and plans
- * with timing on always run eagerly.  Changing tolerances or the Thomas
+ * identical to the eager launch sequence.  A default stream cannot be captured:
+ * solves called on it are captured on a stream of the plan's and the graph is
+ * launched on the caller's.  Plans with timing on always run eagerly.  Changing tolerances or the Thomas
  * configuration drops the captured graph.  on: 0 off, nonzero on. */
 fdi_status fdi_plan_set_graphs(fdi_plan* plan, int on);
 

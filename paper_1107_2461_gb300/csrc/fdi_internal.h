@@ -185,6 +185,7 @@ struct fdi_plan {
     unsigned long long last_use = 0;
   };
   GraphSlot gslots[kGraphSlots];
+  cudaStream_t gstream = nullptr;   // captures the solves called on a default stream (made when needed)
   unsigned long long gclock = 0;
   // host-buffer solves (fdi_field_solve_host): device staging for two
   // right-hand sides and two solutions, copy streams and their events, and

@@ -275,6 +275,7 @@ void free_plan(fdi_plan* p) {
   }
   if (p->sfork) cudaEventDestroy(p->sfork);
   if (p->cstream) cudaStreamDestroy(p->cstream);
+  if (p->gstream) cudaStreamDestroy(p->gstream);
   free_workspace(p);
   for (double* w : p->sk)
     if (w) cudaFree(w);
