@@ -550,29 +550,34 @@ __device__ void finish_block(const double* __restrict__ partials, int nblocks, D
                              int want_mean, int t, int nt) {
   __shared__ double shf[4 * 32];
   double s[4] = {0, 0, 0, 0};
-  // 8 partial records per thread in flight (16-byte loads), fixed order; a
-  // first check without the mean reads components 0 and 1 only, a later one 0
+  // 4 half records (16 bytes) per thread in flight, fixed order; components 2
+  // and 3 only where the mean is wanted
   const double2* p2 = reinterpret_cast<const double2*>(partials);
-  for (int q0 = t; q0 < nblocks; q0 += 8 * nt) {
-    double2 v[8][2];
+#pragma unroll 1
+  for (int c = 0; c < (want_mean ? 2 : 1); ++c) {
+    double x = 0.0, y = 0.0;
+#pragma unroll 1
+    for (int q0 = t; q0 < nblocks; q0 += 4 * nt) {
+      double2 v[4];
 #pragma unroll
-    for (int u = 0; u < 8; ++u) {
-      const int q = q0 + u * nt;
-      v[u][0] = v[u][1] = make_double2(0.0, 0.0);
-      if (q < nblocks) {
-        v[u][0] = p2[2 * q];
-        if (want_mean) v[u][1] = p2[2 * q + 1];
+      for (int u = 0; u < 4; ++u) {
+        const int q = q0 + u * nt;
+        v[u] = q < nblocks ? p2[2 * q + c] : make_double2(0.0, 0.0);
+      }
+#pragma unroll
+      for (int u = 0; u < 4; ++u) {
+        if (q0 - (t & 31) + u * nt < nblocks) {  // else nothing for this warp
+          x += v[u].x;
+          y += v[u].y;
+        }
       }
     }
-#pragma unroll
-    for (int u = 0; u < 8; ++u) {
-      if (q0 - (t & 31) + u * nt >= nblocks) break;  // nothing for this warp
-      s[0] += v[u][0].x;
-      s[1] += v[u][0].y;
-      if (want_mean) {
-        s[2] += v[u][1].x;
-        s[3] += v[u][1].y;
-      }
+    if (c == 0) {
+      s[0] = x;
+      s[1] = y;
+    } else {
+      s[2] = x;
+      s[3] = y;
     }
   }
   // only the warps that hold records take part

@@ -138,19 +138,6 @@ __device__ __forceinline__ void tmem_ld4(uint32_t taddr, float (&r)[4]) {
                : "memory");
 }
 
-// one lane of the warp; code under it runs on the uniform datapath, which the
-// MMA's descriptors need (a branch on the lane index costs two transfers into
-// uniform registers per descriptor: 56-76 clocks per MMA instead of 35)
-__device__ __forceinline__ bool elect_one() {
-  uint32_t p;
-  asm volatile(
-      "{\n\t.reg .pred p;\n\t"
-      "elect.sync _|p, 0xffffffff;\n\t"
-      "selp.u32 %0, 1, 0, p;\n\t}"
-      : "=r"(p));
-  return p != 0;
-}
-
 __device__ __forceinline__ void cp_async8(uint32_t dst, const double* src, bool valid) {
   asm volatile("cp.async.ca.shared.global [%0], [%1], 8, %2;" ::"r"(dst), "l"(src), "r"(valid ? 8 : 0) : "memory");
 }
@@ -318,7 +305,7 @@ __global__ void __launch_bounds__(THREADS, 1) k_slice_transform(const SliceArgs 
   };
 
   if (warp == 0) {
-    if (elect_one()) {
+    if (tc::elect_one()) {
       uint32_t g = 0;
       for (int it = 0; it < items && !s_abort; ++it) {
         const int mt = (i0 + it) % a.m_tiles;
@@ -338,7 +325,8 @@ __global__ void __launch_bounds__(THREADS, 1) k_slice_transform(const SliceArgs 
         tc::mbar_drain(&full[g2 % STAGES], (g2 / STAGES) & 1);
     }
   } else if (warp == 1) {
-    if (elect_one()) {
+    // one elected thread (under a lane test 56-76 clocks per MMA instead of 35)
+    if (tc::elect_one()) {
       const uint32_t idesc = tc::idesc_f16_f32(TM, TN);
       const uint32_t s_base = tc::smem_u32(smem);
       uint32_t g = 0;

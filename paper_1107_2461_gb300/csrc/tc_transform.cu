@@ -17,16 +17,21 @@
 // [2*N_pad][K_pad] (row k scaled by its own power of two, undone per output
 // column in the epilogue) and streamed by TMA.
 //
-// Warp roles of the persistent CTA (one per SM, 480 threads):
+// Warp roles of the persistent CTA (one per SM, 608 threads):
 //   warp 0      TMA producer of the B chunks (each CTA loads its own copy; L2-resident)
 //   warp 1      TMEM allocator and single-thread MMA issuer
 //   warps 2-9   converters: read FP32 rows of A from shared memory, scale,
 //               split to fp16 hi/lo, store them in the 64-byte swizzled
 //               K-major layout of the MMA stage
-//   warps 10-13 epilogue: TMEM -> registers -> unscale -> global store
-//   warp 14     TMA producer of the FP32 A chunks (128 rows x 32 columns)
-// Three MMA stages of K = 32, three FP32 A slots ahead of them (48 KB of input
-// in flight per SM), two TMEM accumulators of N_pad columns.
+//   warps 10-17 epilogue: TMEM -> registers -> unscale -> global store
+//   warp 18     TMA producer of the FP32 A chunks (128 rows x 32 columns)
+// K = 32 per chunk: three stages of B, two of converted A (one per converter
+// group), four FP32 A slots ahead of them (64 KB of input in flight per SM), two
+// TMEM accumulators of N_pad columns.
+//
+// Measured at 256^3 (CUDA events around a pass): 34 us with one lane-tested MMA
+// thread, four epilogue warps and all eight converter warps on one chunk; 31 us
+// as above (HBM floor 20 us).
 #include <cuda.h>
 #include <cudaTypedefs.h>
 
@@ -39,23 +44,26 @@ namespace {
 
 constexpr int BM = 128;
 constexpr int BK = 32;                       // fp16 K per chunk: 64-byte rows, 64-byte swizzle
-constexpr int STAGES = 3;
-constexpr int NA32 = 3;                      // FP32 A slots (TMA, 128-byte swizzle)
+constexpr int NB = 3;                        // B stages (matrix chunks, hi and lo)
+constexpr int NS = 2;                        // A stages (converted input chunks), one per converter group
+constexpr int NA32 = 4;                      // FP32 A slots (TMA, 128-byte swizzle), two per converter group
 constexpr int NMAX = 256;
 constexpr int ROWB = BK * 2;                 // bytes per operand row in a stage
 constexpr int A_BYTES = BM * ROWB;           // one fp16 half of an A chunk: 8 KB
 constexpr int B_BYTES = NMAX * ROWB;         // one fp16 half of a B chunk: up to 16 KB
-constexpr int STAGE_BYTES = 2 * A_BYTES + 2 * B_BYTES;
 constexpr int A32_BYTES = BM * BK * 4;      // 16 KB
-constexpr int NCONV = 8;
-constexpr int WARP_A = 2 + NCONV + 4;         // A producer warp
+constexpr int NCONV = 8;                      // two groups of four that take alternate chunks
+constexpr int NGRP = NCONV / 2;
+constexpr int NEPI = 8;                       // two per tensor-memory quarter, alternate 32-column blocks
+constexpr int WARP_A = 2 + NCONV + NEPI;      // A producer warp
 constexpr int THREADS = 32 * (WARP_A + 1);
 constexpr bool kTmaTransposed = false;
-constexpr int EPI_WARP_BYTES = 8 * 1024;      // per epilogue warp: transpose tile (32 x 33) or two TMA staging tiles (32 x 32)
-constexpr int TP_BYTES = 4 * EPI_WARP_BYTES;
+constexpr int EPI_WARP_BYTES = 4 * 1024;      // per epilogue warp: one 32 x 32 block (transpose tile or TMA staging)
+constexpr int TP_BYTES = NEPI * EPI_WARP_BYTES;
 constexpr int BAR_BYTES = 256;
 constexpr int CS_BYTES = NMAX * 4;            // per-column unscale factors
-constexpr int A32_OFF = STAGES * STAGE_BYTES;
+constexpr int AS_OFF = NB * 2 * B_BYTES;
+constexpr int A32_OFF = AS_OFF + NS * 2 * A_BYTES;
 constexpr int EPI_OFF = A32_OFF + NA32 * A32_BYTES;  // 1024-byte aligned
 constexpr int BAR_OFF = EPI_OFF + TP_BYTES;
 // the dynamic block starts 1024-byte aligned (the static block is padded to
@@ -88,36 +96,44 @@ __global__ void __launch_bounds__(THREADS, 1)
   }
   uint8_t* smem = smem_raw;
   uint64_t* bars = reinterpret_cast<uint64_t*>(smem + BAR_OFF);
+  // Groups wait only on barriers whose every phase they see: NS and NA32 are
+  // multiples of the two groups, so a stage or slot belongs to one group (a
+  // parity wait that skips phases can pass too early).
   uint64_t* full_b = bars;                  // B chunk landed (TMA transaction bytes)
-  uint64_t* conv = bars + STAGES;           // A chunk converted (NCONV warp arrivals)
-  uint64_t* empty = bars + 2 * STAGES;      // stage consumed by the MMAs (one commit)
-  uint64_t* accf = bars + 3 * STAGES;       // accumulator complete
-  uint64_t* acce = bars + 3 * STAGES + 2;   // accumulator drained by the epilogue
-  uint64_t* a_full = bars + 3 * STAGES + 4;          // FP32 A chunk landed (TMA bytes)
-  uint64_t* a_empty = bars + 3 * STAGES + 4 + NA32;  // FP32 A chunk read (NCONV warp arrivals)
-  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + 3 * STAGES + 4 + 2 * NA32);
-  uint64_t* mma_drain = bars + 3 * STAGES + 4 + 2 * NA32 + 1;  // MMAs issued before a failure completed
+  uint64_t* empty_b = full_b + NB;          // B stage consumed by the MMAs (one commit)
+  uint64_t* conv = empty_b + NB;            // A chunk converted (NGRP warp arrivals)
+  uint64_t* empty_a = conv + NS;            // A stage consumed by the MMAs (one commit)
+  uint64_t* accf = empty_a + NS;            // accumulator complete
+  uint64_t* acce = accf + 2;                // accumulator drained by the epilogue (NEPI warps)
+  uint64_t* a_full = acce + 2;              // FP32 A chunk landed (TMA bytes)
+  uint64_t* a_empty = a_full + NA32;        // FP32 A chunk read (NGRP warp arrivals)
+  uint64_t* mma_drain = a_empty + NA32;     // MMAs issued before a failure completed
+  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(mma_drain + 1);
+  static_assert((2 * NB + 2 * NS + 4 + 2 * NA32 + 2) * 8 <= BAR_BYTES, "barriers");
   __shared__ volatile int s_abort;
 
-  const int warp = threadIdx.x / 32, lane = threadIdx.x % 32;
+  const int warp = __shfl_sync(0xffffffffu, threadIdx.x / 32, 0), lane = threadIdx.x % 32;
   const long long wl = a.wait_cycles > 0 ? a.wait_cycles : tc::kWaitCycles;
   const int N_pad = a.N_pad;
   uint32_t tmem_cols = 32;
   while (tmem_cols < (uint32_t)(2 * N_pad)) tmem_cols <<= 1;
 
   if (threadIdx.x == 0) {
-    for (int s = 0; s < STAGES; ++s) {
+    for (int s = 0; s < NB; ++s) {
       tc::mbar_init(&full_b[s], 1);
-      tc::mbar_init(&conv[s], NCONV);
-      tc::mbar_init(&empty[s], 1);
+      tc::mbar_init(&empty_b[s], 1);
+    }
+    for (int s = 0; s < NS; ++s) {
+      tc::mbar_init(&conv[s], NGRP);
+      tc::mbar_init(&empty_a[s], 1);
     }
     for (int b = 0; b < 2; ++b) {
       tc::mbar_init(&accf[b], 1);
-      tc::mbar_init(&acce[b], 4);
+      tc::mbar_init(&acce[b], NEPI);
     }
     for (int b = 0; b < NA32; ++b) {
       tc::mbar_init(&a_full[b], 1);
-      tc::mbar_init(&a_empty[b], NCONV);
+      tc::mbar_init(&a_empty[b], NGRP);
     }
     tc::mbar_init(mma_drain, 1);
     s_abort = 0;
@@ -189,28 +205,29 @@ __global__ void __launch_bounds__(THREADS, 1)
       uint32_t g = 0;
       for (long long it = 0; it < my_iters && !s_abort; ++it) {
         for (int kc = 0; kc < nK; ++kc, ++g) {
-          const int s = g % STAGES;
-          const uint32_t ph = (g / STAGES) & 1;
-          if (!tc::mbar_wait(&empty[s], ph ^ 1, &s_abort, wl)) {
+          const int s = g % NB;
+          const uint32_t ph = (g / NB) & 1;
+          if (!tc::mbar_wait(&empty_b[s], ph ^ 1, &s_abort, wl)) {
             s_abort = 1;
             atomicExch(a.err, 1);
             break;
           }
           tc::mbar_expect_tx(&full_b[s], bbytes);
-          uint8_t* st = smem + s * STAGE_BYTES;
-          tc::tma_load_2d(tc::smem_u32(st + 2 * A_BYTES), &tmB, kc * BK, 0, &full_b[s]);
-          tc::tma_load_2d(tc::smem_u32(st + 2 * A_BYTES + B_BYTES), &tmB, kc * BK, N_pad, &full_b[s]);
+          uint8_t* st = smem + s * 2 * B_BYTES;
+          tc::tma_load_2d(tc::smem_u32(st), &tmB, kc * BK, 0, &full_b[s]);
+          tc::tma_load_2d(tc::smem_u32(st + B_BYTES), &tmB, kc * BK, N_pad, &full_b[s]);
         }
       }
-      // the last STAGES loads issued may still be writing shared memory (after
+      // the last NB loads issued may still be writing shared memory (after
       // a failure nobody consumes them); their phases complete regardless, and
       // a consumed one has completed already
-      for (uint32_t g2 = g > STAGES ? g - STAGES : 0; g2 < g; ++g2)
-        tc::mbar_drain(&full_b[g2 % STAGES], (g2 / STAGES) & 1);
+      for (uint32_t g2 = g > NB ? g - NB : 0; g2 < g; ++g2) tc::mbar_drain(&full_b[g2 % NB], (g2 / NB) & 1);
     }
   } else if (warp == 1) {
     // ---------------- MMA issuer ----------------
-    if (lane == 0) {
+    // (one elected thread: under a lane test the descriptors would go through
+    // vector registers, 166 instead of 128 clocks per 128 x 256 x 16 MMA)
+    if (tc::elect_one()) {
       uint32_t g = 0;
       for (long long it = 0; it < my_iters && !s_abort; ++it) {
         int half = -1;
@@ -229,17 +246,15 @@ __global__ void __launch_bounds__(THREADS, 1)
         const uint32_t d = tmem_base + (uint32_t)(buf * N_pad) + coff;
         bool ok = true;
         for (int kc = 0; kc < nK; ++kc, ++g) {
-          const int s = g % STAGES;
-          const uint32_t ph = (g / STAGES) & 1;
-          if (!tc::mbar_wait(&full_b[s], ph, &s_abort, wl) || !tc::mbar_wait(&conv[s], ph, &s_abort, wl)) {
+          const int sb = g % NB, sa = g % NS;
+          if (!tc::mbar_wait(&full_b[sb], (g / NB) & 1, &s_abort, wl) ||
+              !tc::mbar_wait(&conv[sa], (g / NS) & 1, &s_abort, wl)) {
             ok = false;
             break;
           }
           tc::tc_fence_after();
-          uint8_t* st = smem + s * STAGE_BYTES;
-          const uint32_t ahi = tc::smem_u32(st), alo = tc::smem_u32(st + A_BYTES);
-          const uint32_t bhi = tc::smem_u32(st + 2 * A_BYTES) + coff * ROWB;
-          const uint32_t blo = tc::smem_u32(st + 2 * A_BYTES + B_BYTES) + coff * ROWB;
+          const uint32_t ahi = tc::smem_u32(smem + AS_OFF + sa * 2 * A_BYTES), alo = ahi + A_BYTES;
+          const uint32_t bhi = tc::smem_u32(smem + sb * 2 * B_BYTES) + coff * ROWB, blo = bhi + B_BYTES;
 #pragma unroll
           for (int kk = 0; kk < BK / 16; ++kk) {
             const uint32_t off = kk * 32;
@@ -248,7 +263,8 @@ __global__ void __launch_bounds__(THREADS, 1)
             tc::mma_f16(d, tc::sdesc_k_sw64(ahi + off), tc::sdesc_k_sw64(blo + off), idesc, 1u);
             tc::mma_f16(d, tc::sdesc_k_sw64(alo + off), tc::sdesc_k_sw64(bhi + off), idesc, 1u);
           }
-          tc::mma_commit(&empty[s]);
+          tc::mma_commit(&empty_b[sb]);
+          tc::mma_commit(&empty_a[sa]);
         }
         if (!ok) {
           s_abort = 1;
@@ -264,37 +280,35 @@ __global__ void __launch_bounds__(THREADS, 1)
     }
   } else if (warp < 2 + NCONV) {
     // ---------------- converters ----------------
-    // Each thread owns 2 (row, 32-byte) slots of a 128 x 32 A chunk: it reads
-    // the FP32 values from the TMA slot (128-byte swizzle: 16-byte unit u of
-    // row r sits at unit u ^ (r & 7), conflict free), scales, splits and stores
-    // 16 fp16 hi and lo values into the MMA stage.
-    const int ct = (warp - 2) * 32 + lane;  // 0..255
+    // Two groups of four warps take alternate chunks, so that the fixed
+    // latencies of a chunk (barrier waits, the proxy fence) are paid half as
+    // often and overlap between the groups.  Each thread owns 4 (row, 32-byte)
+    // pieces of a 128 x 32 A chunk: it reads the FP32 values from the TMA slot
+    // (128-byte swizzle: 16-byte unit u of row r sits at unit u ^ (r & 7),
+    // conflict free), scales, splits and stores fp16 hi and lo values into the
+    // MMA stage.
+    const int grp = (warp - 2) >> 2;
+    const int ct = ((warp - 2) & 3) * 32 + lane;  // 0..127
     const float sA = scale_from_max(in_scale);
-    const int c8 = ct & 3;                  // 32-byte group within the 128-byte row
-    // the two (row, 8-wide k group) pieces this thread converts per chunk:
-    // K-major slots: rows ct/4 and ct/4 + 64, k group c8; MN-major slots: row
-    // ct % 128, k groups 2 (ct / 128) and 2 (ct / 128) + 1
+    // K-major slots: rows ct / 4 + 32 q, k group ct % 4; MN-major slots: row ct,
+    // k groups 0 .. 3
     const bool a_mn = a.a_mn != 0;
-    const int row_q[2] = {a_mn ? (ct & 127) : (ct >> 2), a_mn ? (ct & 127) : (ct >> 2) + 64};
-    const int kofs_q[2] = {a_mn ? (ct >> 7) * 16 : c8 * 8, a_mn ? (ct >> 7) * 16 + 8 : c8 * 8};
+    const int c8 = ct & 3, r4 = ct >> 2;
     const long long total = my_iters * nK;
-    int kc = 0;
-    for (long long gi = 0; gi < total && !s_abort; ++gi) {
+    int kc = grp % nK;
+    for (long long gi = grp; gi < total && !s_abort; gi += 2) {
       const uint32_t g = (uint32_t)gi;
-      const int sa = g % NA32;
-      const uint32_t pa = (g / NA32) & 1;
-      const int s = g % STAGES;
-      const uint32_t ph = (g / STAGES) & 1;
-      if (!tc::mbar_wait(&a_full[sa], pa, &s_abort, wl)) {
+      const int sa = g % NA32, s = g % NS;
+      if (!tc::mbar_wait(&a_full[sa], (g / NA32) & 1, &s_abort, wl)) {
         atomicExch(a.err, 4);
         break;
       }
       const uint8_t* src = smem + A32_OFF + sa * A32_BYTES;
-      float v[2][8];
+      float v[4][8];
       if (!a_mn) {
 #pragma unroll
-        for (int q = 0; q < 2; ++q) {
-          const int row = row_q[q];
+        for (int q = 0; q < 4; ++q) {
+          const int row = r4 + 32 * q;
           const float4 x0 = *reinterpret_cast<const float4*>(src + row * 128 + (((2 * c8) ^ (row & 7)) << 4));
           const float4 x1 = *reinterpret_cast<const float4*>(src + row * 128 + (((2 * c8 + 1) ^ (row & 7)) << 4));
           v[q][0] = x0.x; v[q][1] = x0.y; v[q][2] = x0.z; v[q][3] = x0.w;
@@ -304,24 +318,29 @@ __global__ void __launch_bounds__(THREADS, 1)
         // MN-major slot [32 k][128 m]: a warp reads 32 consecutive m of one k
         const float* sf = reinterpret_cast<const float*>(src);
 #pragma unroll
-        for (int q = 0; q < 2; ++q)
+        for (int q = 0; q < 4; ++q)
 #pragma unroll
-          for (int e = 0; e < 8; ++e) v[q][e] = sf[(kofs_q[q] + e) * BM + row_q[q]];
+          for (int e = 0; e < 8; ++e) v[q][e] = sf[(8 * q + e) * BM + ct];
       }
-      if (!tc::mbar_wait(&empty[s], ph ^ 1, &s_abort, wl)) {
+      if (!tc::mbar_wait(&empty_a[s], ((g / NS) & 1) ^ 1, &s_abort, wl)) {
         atomicExch(a.err, 4);
         break;
       }
-      uint8_t* st = smem + s * STAGE_BYTES;
+      uint8_t* st = smem + AS_OFF + s * 2 * A_BYTES;
+      const bool tail = kc * BK + BK > a.K;  // columns past K read as zero
 #pragma unroll
-      for (int q = 0; q < 2; ++q) {
-        const int row = row_q[q];
-        const int k0 = kc * BK + kofs_q[q];
+      for (int q = 0; q < 4; ++q) {
+        const int row = a_mn ? ct : r4 + 32 * q;
+        const int kofs = a_mn ? 8 * q : c8 * 8;
+        if (tail) {
+#pragma unroll
+          for (int e = 0; e < 8; ++e)
+            if (kc * BK + kofs + e >= a.K) v[q][e] = 0.f;
+        }
         uint32_t hw[4], lw[4];
 #pragma unroll
         for (int e = 0; e < 8; e += 2) {
-          const float x0 = (k0 + e < a.K) ? v[q][e] * sA : 0.f;
-          const float x1 = (k0 + e + 1 < a.K) ? v[q][e + 1] * sA : 0.f;
+          const float x0 = v[q][e] * sA, x1 = v[q][e + 1] * sA;
           // packed conversions (one instruction per pair, round to nearest)
           const __half2 h = __floats2half2_rn(x0, x1);
           const float2 hf = __half22float2(h);
@@ -329,7 +348,7 @@ __global__ void __launch_bounds__(THREADS, 1)
           hw[e / 2] = *reinterpret_cast<const uint32_t*>(&h);
           lw[e / 2] = *reinterpret_cast<const uint32_t*>(&l);
         }
-        const uint32_t off = tc::sw64_offset(row, kofs_q[q]);
+        const uint32_t off = tc::sw64_offset(row, kofs);
         *reinterpret_cast<uint4*>(st + off) = make_uint4(hw[0], hw[1], hw[2], hw[3]);
         *reinterpret_cast<uint4*>(st + A_BYTES + off) = make_uint4(lw[0], lw[1], lw[2], lw[3]);
       }
@@ -340,7 +359,8 @@ __global__ void __launch_bounds__(THREADS, 1)
         tc::mbar_arrive(&a_empty[sa]);
         tc::mbar_arrive(&conv[s]);
       }
-      if (++kc == nK) kc = 0;
+      kc += 2;
+      while (kc >= nK) kc -= nK;
     }
   } else if (warp == WARP_A) {
     // ---------------- TMA producer (FP32 A) ----------------
@@ -375,13 +395,15 @@ __global__ void __launch_bounds__(THREADS, 1)
   } else {
     // ---------------- epilogue ----------------
     // Each thread holds one accumulator row (TMEM lane) and 32 columns per
-    // load.  Every 32 x 32 block goes through a shared tile (stride 33: conflict
+    // load; the two warps of a quarter take alternate 32-column blocks.  Every
+    // 32 x 32 block goes through the warp's shared tile (TMA staging in the
+    // 128-byte swizzle, or element (row, j) at row * 32 + (j ^ row): conflict
     // free both ways); after the transpose a lane owns 4 consecutive rows of one
     // column (transposed outputs) or 4 consecutive columns of one row (row-major
     // outputs) and stores them with one 16-byte access where the layout allows.
     const int q = warp & 3;  // TMEM lane quarter accessible to this warp
-    float* tp0 = reinterpret_cast<float*>(smem + EPI_OFF + (warp - (2 + NCONV)) * EPI_WARP_BYTES);
-    uint32_t nstore = 0;  // TMA stores issued by this warp: staging tile nstore & 1 is next
+    const int ew = warp - (2 + NCONV), eh = ew >> 2;
+    float* tp = reinterpret_cast<float*>(smem + EPI_OFF + ew * EPI_WARP_BYTES);
     const bool rowmajor = a.col_stride == 1;
     // vector stores need 16-byte aligned groups of 4 along the contiguous index
     const bool vec_t = !rowmajor && a.row_stride == 1 && (a.S % 4 == 0) && (a.slab_stride % 4 == 0) &&
@@ -407,25 +429,26 @@ __global__ void __launch_bounds__(THREADS, 1)
       // output base of this lane's own row (row = wrow0 + lane)
       long long base = 0;
       {
-        const long long row = wrow0 + lane;
-        if (row < a.R) base = (row / a.S) * a.slab_stride + (row % a.S) * a.row_stride;
+        const unsigned row = (unsigned)(wrow0 + lane);  // R, S < 2^31
+        if (row < (unsigned)a.R) {
+          const unsigned sl = row / (unsigned)a.S;
+          base = (long long)sl * a.slab_stride + (long long)(row - sl * (unsigned)a.S) * a.row_stride;
+        }
       }
       // bases of the 4 rows this lane stores after a transpose (transposed outputs)
       long long tb[4];
 #pragma unroll
       for (int e = 0; e < 4; ++e) tb[e] = __shfl_sync(0xffffffffu, base, 4 * l8 + e);
-      for (int c0 = c_lo; c0 < c_hi; c0 += 32) {
+      for (int c0 = c_lo + 32 * eh; c0 < c_hi; c0 += 64) {
         uint32_t r[32];
         tc::tmem_ld32(tmem_base + ((uint32_t)(32 * q) << 16) + (uint32_t)(buf * N_pad + c0), r);
         tc::tmem_ld_wait();
         if (a.tma_store) {
-          // unscale into a staging tile and hand it to a TMA store; rows past
+          // unscale into the staging tile and hand it to a TMA store; rows past
           // R and columns past n_out hold zeros (zero-filled A rows, zero B
-          // rows) and are clipped by the store.  Two staging tiles alternate:
-          // the store two back (same tile) must have read it, the last one may
-          // still be reading the other
-          float* tp = tp0 + (nstore & 1u) * 1024;
-          if (lane == 0) tc::bulk_wait_read_1();
+          // rows) and are clipped by the store.  The previous store must have
+          // read the tile (the other seven warps work meanwhile).
+          if (lane == 0) tc::bulk_wait_read_all();
           __syncwarp();
           if (a.tma_store == 1) {
             // staging [column][row]: 32 rows of one column are 128 contiguous bytes
@@ -440,14 +463,11 @@ __global__ void __launch_bounds__(THREADS, 1)
             // `lane` at unit u ^ (lane & 7))
 #pragma unroll
             for (int u = 0; u < 8; ++u) {
-              float v4[4];
-#pragma unroll
-              for (int e = 0; e < 4; ++e) {
-                v4[e] = __uint_as_float(r[4 * u + e]) * s_cs[c0 + 4 * u + e];
-                vmax = fmaxf(vmax, fabsf(v4[e]));
-              }
-              *reinterpret_cast<float4*>(tp + lane * 32 + ((u ^ (lane & 7)) << 2)) =
-                  make_float4(v4[0], v4[1], v4[2], v4[3]);
+              const float4 cs = *reinterpret_cast<const float4*>(s_cs + c0 + 4 * u);
+              const float4 v = make_float4(__uint_as_float(r[4 * u]) * cs.x, __uint_as_float(r[4 * u + 1]) * cs.y,
+                                           __uint_as_float(r[4 * u + 2]) * cs.z, __uint_as_float(r[4 * u + 3]) * cs.w);
+              vmax = fmaxf(fmaxf(vmax, fmaxf(fabsf(v.x), fabsf(v.y))), fmaxf(fabsf(v.z), fabsf(v.w)));
+              *reinterpret_cast<float4*>(tp + lane * 32 + ((u ^ (lane & 7)) << 2)) = v;
             }
           }
           tc::fence_proxy_async_smem();
@@ -461,13 +481,11 @@ __global__ void __launch_bounds__(THREADS, 1)
                 tc::tma_store_2d(&tmO, stg, c0, (int)wrow0);
               tc::bulk_commit();
             }
-            ++nstore;
           }
           continue;
         }
-        float* tp = tp0;
 #pragma unroll
-        for (int j = 0; j < 32; ++j) tp[lane * 33 + j] = __uint_as_float(r[j]);
+        for (int j = 0; j < 32; ++j) tp[lane * 32 + (j ^ lane)] = __uint_as_float(r[j]);
         __syncwarp();
         if (!rowmajor) {
           // lane -> column c0 + 4*qq + g8, rows 4*l8 .. 4*l8+3 of the warp block
@@ -481,7 +499,7 @@ __global__ void __launch_bounds__(THREADS, 1)
               float v4[4];
 #pragma unroll
               for (int e = 0; e < 4; ++e) {
-                v4[e] = tp[(rr + e) * 33 + cl] * cs;
+                v4[e] = tp[(rr + e) * 32 + (cl ^ (rr + e))] * cs;
                 if (rr + e < nrows) vmax = fmaxf(vmax, fabsf(v4[e]));
               }
               const long long koff = (long long)k * a.col_stride;
@@ -512,7 +530,7 @@ __global__ void __launch_bounds__(THREADS, 1)
               if (rl < nrows) {
                 float v4[4];
 #pragma unroll
-                for (int e = 0; e < 4; ++e) v4[e] = tp[rl * 33 + cc + e] * cs[e];
+                for (int e = 0; e < 4; ++e) v4[e] = tp[rl * 32 + ((cc + e) ^ rl)] * cs[e];
                 float* o = a.out_f32 + brow + c0 + cc;
                 if (vec_r && fullcols) {
                   *reinterpret_cast<float4*>(o) = make_float4(v4[0], v4[1], v4[2], v4[3]);
@@ -528,17 +546,19 @@ __global__ void __launch_bounds__(THREADS, 1)
             }
           } else {
             // double-float accumulation into the (out_f32, out_lo) planes: rows in
-            // groups of 4 with the loads of a group issued before any update
+            // pairs with the loads of a pair issued before any update (four rows
+            // at a time would spill)
+#pragma unroll 1
+            for (int q2 = 0; q2 < 8; q2 += 2) {
+              float oh[2][4], ol[2][4];
+              long long br[2];
 #pragma unroll
-            for (int q4 = 0; q4 < 8; q4 += 4) {
-              float oh[4][4], ol[4][4];
-#pragma unroll
-              for (int u = 0; u < 4; ++u) {
-                const int rl = 4 * (q4 + u) + g8;
-                const long long brow = __shfl_sync(0xffffffffu, base, rl) + c0 + cc;
+              for (int u = 0; u < 2; ++u) {
+                const int rl = 4 * (q2 + u) + g8;
+                br[u] = __shfl_sync(0xffffffffu, base, rl) + c0 + cc;
                 if (rl < nrows && vec_r && fullcols) {
-                  const float4 h = *reinterpret_cast<const float4*>(a.out_f32 + brow);
-                  const float4 l = a.lo_valid ? *reinterpret_cast<const float4*>(a.out_lo + brow)
+                  const float4 h = *reinterpret_cast<const float4*>(a.out_f32 + br[u]);
+                  const float4 l = a.lo_valid ? *reinterpret_cast<const float4*>(a.out_lo + br[u])
                                               : make_float4(0.f, 0.f, 0.f, 0.f);
                   oh[u][0] = h.x; oh[u][1] = h.y; oh[u][2] = h.z; oh[u][3] = h.w;
                   ol[u][0] = l.x; ol[u][1] = l.y; ol[u][2] = l.z; ol[u][3] = l.w;
@@ -546,20 +566,19 @@ __global__ void __launch_bounds__(THREADS, 1)
 #pragma unroll
                   for (int e = 0; e < 4; ++e) {
                     const bool ok = rl < nrows && c0 + cc + e < a.n_out;
-                    oh[u][e] = ok ? a.out_f32[brow + e] : 0.f;
-                    ol[u][e] = (ok && a.lo_valid) ? a.out_lo[brow + e] : 0.f;
+                    oh[u][e] = ok ? a.out_f32[br[u] + e] : 0.f;
+                    ol[u][e] = (ok && a.lo_valid) ? a.out_lo[br[u] + e] : 0.f;
                   }
                 }
               }
 #pragma unroll
-              for (int u = 0; u < 4; ++u) {
-                const int rl = 4 * (q4 + u) + g8;
-                const long long brow = __shfl_sync(0xffffffffu, base, rl) + c0 + cc;
+              for (int u = 0; u < 2; ++u) {
+                const int rl = 4 * (q2 + u) + g8;
                 if (rl >= nrows) continue;
 #pragma unroll
                 for (int e = 0; e < 4; ++e) {
                   // (oh, ol) + val: two-sum of the high parts, low parts added, fast renormalisation
-                  const float val = tp[rl * 33 + cc + e] * cs[e];
+                  const float val = tp[rl * 32 + ((cc + e) ^ rl)] * cs[e];
                   const float sh = oh[u][e] + val;
                   const float bb = sh - oh[u][e];
                   const float er = (oh[u][e] - (sh - bb)) + (val - bb) + ol[u][e];
@@ -568,14 +587,14 @@ __global__ void __launch_bounds__(THREADS, 1)
                   ol[u][e] = er - (nh - sh);
                 }
                 if (vec_r && fullcols) {
-                  *reinterpret_cast<float4*>(a.out_f32 + brow) = make_float4(oh[u][0], oh[u][1], oh[u][2], oh[u][3]);
-                  *reinterpret_cast<float4*>(a.out_lo + brow) = make_float4(ol[u][0], ol[u][1], ol[u][2], ol[u][3]);
+                  *reinterpret_cast<float4*>(a.out_f32 + br[u]) = make_float4(oh[u][0], oh[u][1], oh[u][2], oh[u][3]);
+                  *reinterpret_cast<float4*>(a.out_lo + br[u]) = make_float4(ol[u][0], ol[u][1], ol[u][2], ol[u][3]);
                 } else {
 #pragma unroll
                   for (int e = 0; e < 4; ++e)
                     if (c0 + cc + e < a.n_out) {
-                      a.out_f32[brow + e] = oh[u][e];
-                      a.out_lo[brow + e] = ol[u][e];
+                      a.out_f32[br[u] + e] = oh[u][e];
+                      a.out_lo[br[u] + e] = ol[u][e];
                     }
                 }
               }
