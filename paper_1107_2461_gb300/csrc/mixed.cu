@@ -42,9 +42,6 @@ struct MixedAxis {
   float2* wm = nullptr;
   float2* w0 = nullptr;
   float2* m_df = nullptr; // control-volume widths in double-float
-  // resident solve (n <= 128): fwd and bwd in the shared-memory layout of its
-  // MMAs (see tc_resident_image)
-  uint8_t* rimg[2] = {nullptr, nullptr};
 };
 
 namespace {
@@ -881,10 +878,6 @@ fdi_status setup_axis(fdi_plan* p, Axis* ax, cudaStream_t s) {
   const int n = ax->n;
   FDI_TRY(tc_prepare_matrix(p, ax->Einv, n, &mx->fwd, s));
   FDI_TRY(tc_prepare_matrix(p, ax->E, n, &mx->bwd, s));
-  if (n <= kResMaxPlane) {
-    FDI_TRY(tc_resident_image(p, mx->fwd, &mx->rimg[0], s));
-    FDI_TRY(tc_resident_image(p, mx->bwd, &mx->rimg[1], s));
-  }
   FDI_TRY(upload_f(&mx->m_f, ax->h_m));
   FDI_TRY(upload_f(&mx->kd_f, ax->h_kd));
   FDI_TRY(upload_f(&mx->ko_f, ax->h_ko));
@@ -910,7 +903,7 @@ void mixed_free_axis(Axis* ax) {
   if (!mx) return;
   tc_free_matrix(&mx->fwd);
   tc_free_matrix(&mx->bwd);
-  void* ptrs[] = {mx->m_f, mx->kd_f, mx->ko_f, mx->wp, mx->wm, mx->w0, mx->m_df, mx->rimg[0], mx->rimg[1]};
+  void* ptrs[] = {mx->m_f, mx->kd_f, mx->ko_f, mx->wp, mx->wm, mx->w0, mx->m_df};
   for (void* q : ptrs)
     if (q) cudaFree(q);
   delete mx;
@@ -981,8 +974,6 @@ bool resident_eligible(const fdi_plan* p, int field) {
   if (field < 0 || field >= p->nfields || !p->res_bar) return false;
   const Field& f = p->fields[field];
   if (f.n[0] > kResMaxPlane || f.n[1] > kResMaxPlane) return false;
-  for (int d = 0; d < 2; ++d)
-    if (!static_cast<const MixedAxis*>(f.ax[d]->mixed)->rimg[0]) return false;
   return true;
 }
 
@@ -1024,10 +1015,10 @@ fdi_status resident_describe(fdi_plan* p, int field, double sigma, double lambda
   const MixedAxis* mz = static_cast<const MixedAxis*>(f.ax[2]->mixed);
   J.kx = (J.nx + 31) / 32;
   J.ky = (J.ny + 31) / 32;
-  J.img[0][0] = mx->rimg[0];
-  J.img[0][1] = my->rimg[0];
-  J.img[1][0] = mx->rimg[1];
-  J.img[1][1] = my->rimg[1];
+  J.img[0][0] = mx->fwd.img;
+  J.img[0][1] = my->fwd.img;
+  J.img[1][0] = mx->bwd.img;
+  J.img[1][1] = my->bwd.img;
   J.csc[0][0] = mx->fwd.col_scale;
   J.csc[0][1] = my->fwd.col_scale;
   J.csc[1][0] = mx->bwd.col_scale;

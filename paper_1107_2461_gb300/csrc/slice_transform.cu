@@ -147,13 +147,6 @@ __device__ __forceinline__ void cp_async_wait() {
   asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory");
 }
 
-// untiled bulk copy global -> shared (16-byte aligned), counted on an mbarrier
-__device__ __forceinline__ void bulk_load(uint32_t dst, const void* src, uint32_t bytes, uint64_t* bar) {
-  asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(dst),
-               "l"(src), "r"(bytes), "r"(tc::smem_u32(bar))
-               : "memory");
-}
-
 // x = +-m 2^(e - 1075) on a line whose largest biased exponent is eb, as the
 // fixed-point number round(x 2^(62 - (eb - 1022))), |.| < 2^62, plus 128 in every
 // base-256 digit: byte q of the result is digit 7 - q plus 128
@@ -317,7 +310,7 @@ __global__ void __launch_bounds__(THREADS, 1) k_slice_transform(const SliceArgs 
             break;
           }
           tc::mbar_expect_tx(&full[s], A_BYTES);
-          bulk_load(tc::smem_u32(smem + s * SM::STAGE_BYTES), src + (size_t)kc * A_BYTES, A_BYTES, &full[s]);
+          tc::bulk_load(tc::smem_u32(smem + s * SM::STAGE_BYTES), src + (size_t)kc * A_BYTES, A_BYTES, &full[s]);
         }
       }
       // copies issued last may still be writing shared memory after a failure

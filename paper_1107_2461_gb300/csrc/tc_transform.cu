@@ -13,12 +13,13 @@
 // Data layout: the input field is a row-major [R][pitch] FP32 matrix with the
 // contraction index contiguous; the pass sequence of the solver writes each
 // intermediate field in the orientation the next pass reads (see mixed.cu).
-// The transform matrix T is split at plan time into B = [T_hi; T_lo] fp16
-// [2*N_pad][K_pad] (row k scaled by its own power of two, undone per output
-// column in the epilogue) and streamed by TMA.
+// The transform matrix T is split at plan time into B = [T_hi; T_lo] fp16 (row k
+// scaled by its own power of two, undone per output column in the epilogue),
+// stored chunk by chunk in the MMA's shared-memory layout, and streamed by bulk
+// copies.
 //
 // Warp roles of the persistent CTA (one per SM, 608 threads):
-//   warp 0      TMA producer of the B chunks (each CTA loads its own copy; L2-resident)
+//   warp 0      producer of the B chunks (each CTA loads its own copy; L2-resident)
 //   warp 1      TMEM allocator and single-thread MMA issuer
 //   warps 2-9   converters: read FP32 rows of A from shared memory, scale,
 //               split to fp16 hi/lo, store them in the 64-byte swizzled
@@ -84,8 +85,7 @@ __device__ __forceinline__ float scale_from_max(float mx) {
 
 
 __global__ void __launch_bounds__(THREADS, 1)
-    k_tc_transform(const __grid_constant__ CUtensorMap tmB, const __grid_constant__ CUtensorMap tmA,
-                   const __grid_constant__ CUtensorMap tmO, TcArgs a) {
+    k_tc_transform(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmO, TcArgs a) {
   extern __shared__ __align__(1024) uint8_t smem_raw[];
   // the swizzled layouts need a 1024-byte aligned base; the launch reserves no
   // slack for re-alignment, so a misaligned block reports an error instead
@@ -139,7 +139,6 @@ __global__ void __launch_bounds__(THREADS, 1)
     s_abort = 0;
     tc::fence_mbar_init();
   }
-  if (warp == 0 && lane == 0) tc::prefetch_tmap(&tmB);
   if (warp == WARP_A && lane == 0) tc::prefetch_tmap(&tmA);
   if (warp == 1) {
     tc::tmem_alloc(tmem_slot, tmem_cols);
@@ -199,7 +198,7 @@ __global__ void __launch_bounds__(THREADS, 1)
   const int nK = a.nK;
 
   if (warp == 0) {
-    // ---------------- TMA producer (B) ----------------
+    // ---------------- producer of the B chunks (one bulk copy each) ----------------
     if (lane == 0) {
       const uint32_t bbytes = (uint32_t)(2 * N_pad * ROWB);
       uint32_t g = 0;
@@ -213,9 +212,7 @@ __global__ void __launch_bounds__(THREADS, 1)
             break;
           }
           tc::mbar_expect_tx(&full_b[s], bbytes);
-          uint8_t* st = smem + s * 2 * B_BYTES;
-          tc::tma_load_2d(tc::smem_u32(st), &tmB, kc * BK, 0, &full_b[s]);
-          tc::tma_load_2d(tc::smem_u32(st + B_BYTES), &tmB, kc * BK, N_pad, &full_b[s]);
+          tc::bulk_load(tc::smem_u32(smem + s * 2 * B_BYTES), a.img + (size_t)kc * bbytes, bbytes, &full_b[s]);
         }
       }
       // the last NB loads issued may still be writing shared memory (after
@@ -254,7 +251,7 @@ __global__ void __launch_bounds__(THREADS, 1)
           }
           tc::tc_fence_after();
           const uint32_t ahi = tc::smem_u32(smem + AS_OFF + sa * 2 * A_BYTES), alo = ahi + A_BYTES;
-          const uint32_t bhi = tc::smem_u32(smem + sb * 2 * B_BYTES) + coff * ROWB, blo = bhi + B_BYTES;
+          const uint32_t bhi = tc::smem_u32(smem + sb * 2 * B_BYTES) + coff * ROWB, blo = bhi + N_pad * ROWB;
 #pragma unroll
           for (int kk = 0; kk < BK / 16; ++kk) {
             const uint32_t off = kk * 32;
@@ -428,7 +425,7 @@ __global__ void __launch_bounds__(THREADS, 1)
       const int nrows = tvalid ? (int)max(0LL, min((long long)32, a.R - wrow0)) : 0;
       // output base of this lane's own row (row = wrow0 + lane)
       long long base = 0;
-      {
+      if (!a.tma_store) {
         const unsigned row = (unsigned)(wrow0 + lane);  // R, S < 2^31
         if (row < (unsigned)a.R) {
           const unsigned sl = row / (unsigned)a.S;
@@ -490,7 +487,7 @@ __global__ void __launch_bounds__(THREADS, 1)
         if (!rowmajor) {
           // lane -> column c0 + 4*qq + g8, rows 4*l8 .. 4*l8+3 of the warp block
           const int rr = 4 * l8;
-#pragma unroll
+#pragma unroll 2
           for (int qq = 0; qq < 8; ++qq) {
             const int cl = 4 * qq + g8;
             const int k = c0 + cl;
@@ -523,7 +520,7 @@ __global__ void __launch_bounds__(THREADS, 1)
           }
           const bool fullcols = c0 + cc + 3 < a.n_out;
           if (a.mode == TC_OUT_F32) {
-#pragma unroll
+#pragma unroll 2
             for (int qq = 0; qq < 8; ++qq) {
               const int rl = 4 * qq + g8;
               const long long brow = __shfl_sync(0xffffffffu, base, rl);
@@ -623,9 +620,12 @@ __global__ void __launch_bounds__(THREADS, 1)
   }
 }
 
-__global__ void k_prep_b(const double* __restrict__ T, int n, int N_pad, int K_pad, __half* __restrict__ B,
+// The matrix as the MMA reads it from shared memory: for every K chunk of 32,
+// the hi rows then the lo rows (N_pad each), every row 64 bytes in the 64-byte
+// swizzle layout, so a chunk is one bulk copy.  Row k of T (output k) is scaled
+// by a power of two and split into fp16 hi and lo.
+__global__ void k_prep_b(const double* __restrict__ T, int n, int N_pad, int K_pad, uint8_t* __restrict__ img,
                          float* __restrict__ col_scale) {
-  // row k of T (output k) -> scaled by a power of two, split into fp16 hi/lo
   const int k = blockIdx.x;
   __shared__ double smax[256];
   double mx = 0.0;
@@ -645,8 +645,9 @@ __global__ void k_prep_b(const double* __restrict__ T, int n, int N_pad, int K_p
     double t = (k < n && j < n) ? T[(size_t)k * n + j] * sc : 0.0;
     __half h = __double2half(t);
     __half l = __double2half(t - (double)__half2float(h));
-    B[(size_t)k * K_pad + j] = h;
-    B[(size_t)(N_pad + k) * K_pad + j] = l;
+    uint8_t* c = img + (size_t)(j / BK) * (2 * N_pad * ROWB) + tc::sw64_offset(k, j % BK);
+    *reinterpret_cast<__half*>(c) = h;
+    *reinterpret_cast<__half*>(c + (size_t)N_pad * ROWB) = l;
   }
 }
 
@@ -669,57 +670,18 @@ fdi_status tc_prepare_matrix(fdi_plan* p, const double* T, int n, TcMatrix* m, c
   m->n = n;
   m->N_pad = ((n + 31) / 32) * 32;
   m->K_pad = ((n + BK - 1) / BK) * BK;
-  const size_t elems = (size_t)2 * m->N_pad * m->K_pad;
-  FDI_CUDA_TRY(cudaMalloc(&m->B, elems * sizeof(__half)));
+  FDI_CUDA_TRY(cudaMalloc(&m->img, (size_t)2 * m->N_pad * m->K_pad * sizeof(__half)));
   FDI_CUDA_TRY(cudaMalloc(&m->col_scale, m->N_pad * sizeof(float)));
   FDI_CUDA_TRY(cudaMemsetAsync(m->col_scale, 0, m->N_pad * sizeof(float), s));
-  k_prep_b<<<m->N_pad, 256, 0, s>>>(T, n, m->N_pad, m->K_pad, (__half*)m->B, m->col_scale);
-  FDI_LAUNCH_CHECK(p);
-  auto enc = encode_fn();
-  if (!enc) {
-    set_error("cuTensorMapEncodeTiled entry point unavailable");
-    return FDI_ERR_CUDA;
-  }
-  {
-    // B chunks: N_pad rows x 32 fp16 (one half, hi or lo, of a stage's B operand)
-    cuuint64_t dims[2] = {(cuuint64_t)m->K_pad, (cuuint64_t)(2 * m->N_pad)};
-    cuuint64_t strides[1] = {(cuuint64_t)m->K_pad * sizeof(__half)};
-    cuuint32_t box[2] = {(cuuint32_t)BK, (cuuint32_t)m->N_pad};
-    cuuint32_t estr[2] = {1, 1};
-    CUresult r = enc(reinterpret_cast<CUtensorMap*>(m->tmap), CU_TENSOR_MAP_DATA_TYPE_FLOAT16, 2, m->B, dims,
-                     strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_64B,
-                     CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
-    if (r != CUDA_SUCCESS) {
-      set_error("cuTensorMapEncodeTiled failed for a transform matrix");
-      return FDI_ERR_CUDA;
-    }
-  }
-  return FDI_OK;
-}
-
-// The matrix as the resident solve's MMA reads it from shared memory: for
-// every K chunk of 32, the hi rows then the lo rows (N_pad each), every row 64
-// bytes in the 64-byte swizzle layout; copied into shared memory as it is.
-__global__ void k_res_image(const __half* __restrict__ B, int N_pad, int K_pad, uint8_t* __restrict__ img) {
-  const int half = blockIdx.y, n = blockIdx.x;
-  for (int k = threadIdx.x; k < K_pad; k += blockDim.x) {
-    const size_t off = (size_t)(k / BK) * (2 * N_pad * ROWB) + (size_t)half * N_pad * ROWB + tc::sw64_offset(n, k % BK);
-    *reinterpret_cast<__half*>(img + off) = B[((size_t)half * N_pad + n) * K_pad + k];
-  }
-}
-
-fdi_status tc_resident_image(fdi_plan* p, const TcMatrix& m, uint8_t** img, cudaStream_t s) {
-  const size_t bytes = (size_t)(m.K_pad / BK) * 2 * m.N_pad * ROWB;
-  FDI_CUDA_TRY(cudaMalloc(img, bytes));
-  k_res_image<<<dim3((unsigned)m.N_pad, 2), 128, 0, s>>>((const __half*)m.B, m.N_pad, m.K_pad, *img);
+  k_prep_b<<<m->N_pad, 256, 0, s>>>(T, n, m->N_pad, m->K_pad, m->img, m->col_scale);
   FDI_LAUNCH_CHECK(p);
   return FDI_OK;
 }
 
 void tc_free_matrix(TcMatrix* m) {
-  if (m->B) cudaFree(m->B);
+  if (m->img) cudaFree(m->img);
   if (m->col_scale) cudaFree(m->col_scale);
-  m->B = nullptr;
+  m->img = nullptr;
   m->col_scale = nullptr;
 }
 
@@ -741,8 +703,7 @@ fdi_status launch_kernel(fdi_plan* p, const TcMatrix& m, const CUtensorMap& mapA
     const long long tail = tiles % grid;
     if (tail > 0 && 2 * tail <= grid) a2.n_full = tiles - tail;
   }
-  CUtensorMap map;
-  memcpy(&map, m.tmap, sizeof(CUtensorMap));
+  a2.img = m.img;
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3((unsigned)grid);
   cfg.blockDim = dim3(THREADS);
@@ -753,7 +714,7 @@ fdi_status launch_kernel(fdi_plan* p, const TcMatrix& m, const CUtensorMap& mapA
   attr[0].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr;
   cfg.numAttrs = args.pdl ? 1 : 0;
-  FDI_CUDA_TRY(cudaLaunchKernelEx(&cfg, k_tc_transform, map, mapA, mapO, a2));
+  FDI_CUDA_TRY(cudaLaunchKernelEx(&cfg, k_tc_transform, mapA, mapO, a2));
   FDI_LAUNCH_CHECK(p);
   return FDI_OK;
 }

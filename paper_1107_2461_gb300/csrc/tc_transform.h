@@ -12,14 +12,13 @@ namespace fdi {
 enum { TC_OUT_F32 = 0, TC_OUT_DF_ADD = 1 };
 
 // A transform matrix T (n x n, output index k, input index j) prepared for the
-// tensor cores: B = [hi; lo] fp16 [2*N_pad][K_pad], per-row power-of-two scale
-// undone by col_scale[k], and its TMA descriptor.
+// tensor cores: B = [hi; lo] fp16 in the MMA's shared-memory layout (K chunks of
+// 32: N_pad hi rows, N_pad lo rows, 64-byte swizzle; also what the resident solve
+// copies), per-row power-of-two scale undone by col_scale[k].
 struct TcMatrix {
   int n = 0, N_pad = 0, K_pad = 0;
-  void* B = nullptr;
+  unsigned char* img = nullptr;
   float* col_scale = nullptr;
-  // TMA descriptor of B (boxes of N_pad rows x 32 columns)
-  alignas(64) unsigned char tmap[128];
 };
 
 struct TcArgs {
@@ -57,13 +56,11 @@ struct TcArgs {
   // as two half-width items of N_pad / 2 output columns each
   long long n_full = 0;
   const float* col_scale = nullptr;
+  const unsigned char* img = nullptr;
 };
 
 fdi_status tc_prepare_matrix(fdi_plan* p, const double* T, int n, TcMatrix* m, cudaStream_t s);
 void tc_free_matrix(TcMatrix* m);
-// the matrix in the resident solve's shared-memory layout (K chunks of 32:
-// hi rows, lo rows, 64-byte swizzle); cudaMalloc'ed, the caller frees it
-fdi_status tc_resident_image(fdi_plan* p, const TcMatrix& m, uint8_t** img, cudaStream_t s);
 fdi_status launch_tc_transform(fdi_plan* p, const TcMatrix& m, TcArgs args, const char* name, cudaStream_t s);
 
 }  // namespace fdi
