@@ -127,28 +127,52 @@ __global__ void k_finalize_out(const float* __restrict__ xh, const float* __rest
   }
 }
 
-// end of a first-pass block (8 warps): the components' sums, one lane each, and
-// one atomic for max |b|
+// What the first pass sets up for the later ones: the lambda-scaled
+// double-float flux weights ([3 directions][wp, wm, w0][kMaxN] and, for
+// cylindrical plans, the theta flux weight per radial cell) and zeroes in the
+// scale slots that later passes raise by atomic max (slot 0, the pass's own,
+// is stored by its last block).
+struct SetupArgs {
+  const float2* src[10];
+  int n[10];
+  float2 lambda;
+  float2* lam_w;
+  float* scales;
+  int nscales;
+};
+
+__device__ __forceinline__ void first_pass_setup(const SetupArgs& w) {
+  for (int q = blockIdx.x; q < 10; q += gridDim.x)
+    for (int t = threadIdx.x; t < w.n[q]; t += blockDim.x) {
+      const df::F2 v = df::mul(df::make(w.lambda.x, w.lambda.y), ld2(w.src[q] + t));
+      w.lam_w[q * kMaxN + t] = make_float2(v.hi, v.lo);
+    }
+  if (blockIdx.x == gridDim.x - 1)
+    for (int t = 1 + threadIdx.x; t < w.nscales; t += blockDim.x) w.scales[t] = 0.f;
+}
+
+// end of a first-pass block (8 warps): the components' sums, one lane each;
+// component 0 holds max |b|
 __device__ __forceinline__ void init_block_out(const ResidArgs& a, const double* sh, const float* smax, int nc) {
   if (threadIdx.x >= 32) return;
   const int lane = threadIdx.x;
-  if (lane < 4) {
+  if (lane > 0 && lane < 4) {
     double t = 0.0;
-    if (lane > 0 && lane < nc)
+    if (lane < nc)
       for (int q = 0; q < 8; ++q) t += sh[4 * q + lane];
     a.partials[4 * blockIdx.x + lane] = t;
   }
   float m = lane < 8 ? smax[lane] : 0.f;
 #pragma unroll
   for (int o = 4; o > 0; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
-  if (lane == 0 && m > 0.f) atomicMax(reinterpret_cast<unsigned int*>(a.rmax), __float_as_uint(m));
+  if (lane == 0) a.partials[4 * blockIdx.x] = (double)m;
   __syncwarp();  // the record is written before thread 0 fences and takes the ticket
 }
 
 // r_0 = b: FP64 -> FP32 copy into the padded residual layout, ||b||^2, max |b|
 // and (singular problems) the volume-weighted sums; one warp per x-line
-__global__ void __launch_bounds__(256) k_init_rhs(ResidArgs a) {
-  pdl_wait();
+__global__ void __launch_bounds__(256) k_init_rhs(ResidArgs a, SetupArgs w) {
+  first_pass_setup(w);
   __shared__ double sh[4 * 8];
   __shared__ float smax[8];
   const int nx = a.nx, ny = a.ny, nz = a.nz;
@@ -213,8 +237,8 @@ __global__ void __launch_bounds__(256) k_init_rhs(ResidArgs a) {
 // r_0 = b for unpadded fields without the mean (nx a multiple of 4): flat
 // stream, 8 values per thread and iteration (four 16-byte loads in flight),
 // ||b||^2 and max |b|
-__global__ void __launch_bounds__(256) k_init_rhs_flat(ResidArgs a, long long P) {
-  pdl_wait();
+__global__ void __launch_bounds__(256) k_init_rhs_flat(ResidArgs a, SetupArgs w, long long P) {
+  first_pass_setup(w);
   __shared__ double sh[4 * 8];
   __shared__ float smax[8];
   const int warp = threadIdx.x / 32, lane = threadIdx.x % 32;
@@ -264,33 +288,6 @@ __global__ void __launch_bounds__(256) k_init_rhs_flat(ResidArgs a, long long P)
   finish_if_last(a.fin, threadIdx.x, blockDim.x);
 }
 
-// lambda-scaled double-float flux weights of the three directions
-__global__ void k_scale_weights(const float2* __restrict__ wp0, const float2* __restrict__ wm0,
-                                const float2* __restrict__ w00, int n0, const float2* __restrict__ wp1,
-                                const float2* __restrict__ wm1, const float2* __restrict__ w01, int n1,
-                                const float2* __restrict__ wp2, const float2* __restrict__ wm2,
-                                const float2* __restrict__ w02, int n2, const float2* __restrict__ wc, int nc,
-                                float2 lam, float2* __restrict__ out) {
-  // out layout: [3 directions][3 kinds (p, m, 0)][kMaxN], then (cylindrical
-  // plans, block 9) the theta flux weight per radial cell
-  if (blockIdx.x == 9) {
-    for (int t = threadIdx.x; t < nc; t += blockDim.x) {
-      const df::F2 v = df::mul(df::make(lam.x, lam.y), ld2(wc + t));
-      out[9 * kMaxN + t] = make_float2(v.hi, v.lo);
-    }
-    return;
-  }
-  const int d = blockIdx.x / 3, kind = blockIdx.x % 3;
-  const int n = d == 0 ? n0 : (d == 1 ? n1 : n2);
-  const float2* src = d == 0 ? (kind == 0 ? wp0 : kind == 1 ? wm0 : w00)
-                             : d == 1 ? (kind == 0 ? wp1 : kind == 1 ? wm1 : w01)
-                                      : (kind == 0 ? wp2 : kind == 1 ? wm2 : w02);
-  for (int t = threadIdx.x; t < n; t += blockDim.x) {
-    const df::F2 v = df::mul(df::make(lam.x, lam.y), ld2(src + t));
-    out[(d * 3 + kind) * kMaxN + t] = make_float2(v.hi, v.lo);
-  }
-}
-
 // The last block of a reduction grid to finish (atomic ticket after its
 // partials are visible) runs finish_block and re-arms the ticket counter, so
 // the reduction needs no second launch.  Every block has passed its own skip
@@ -305,6 +302,19 @@ __device__ void finish_if_last(const FinishArgs& f, int t, int nt) {
   __syncthreads();
   if (!amlast) return;
   __threadfence();
+  if (f.max_out) {
+    __shared__ float wmax[32];
+    float m = 0.f;
+    for (unsigned q = t; q < nb; q += nt) m = fmaxf(m, (float)f.partials[4 * q]);
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
+    if ((t & 31) == 0) wmax[t >> 5] = m;
+    __syncthreads();
+    if (t == 0) {
+      for (int q = 1; q < nt / 32; ++q) m = fmaxf(m, wmax[q]);
+      *f.max_out = m;
+    }
+  }
   finish_block(f.partials, (int)nb, f.st, f.tol, f.kind, f.want_mean, t, nt);
   if (t == 0) {
     *f.counter = 0u;
@@ -1134,8 +1144,7 @@ fdi_status mixed_field_solve(fdi_plan* p, int field, double sigma, double lambda
   const MixedAxis* mx = static_cast<const MixedAxis*>(f.ax[0]->mixed);
   const MixedAxis* my = static_cast<const MixedAxis*>(f.ax[1]->mixed);
   const MixedAxis* mz = static_cast<const MixedAxis*>(f.ax[2]->mixed);
-  // (the first pass's reduction resets the solve's status)
-  FDI_CUDA_TRY(cudaMemsetAsync(p->d_scales, 0, (size_t)(kMaxRefineCap + 2) * kScaleStride * sizeof(float), s));
+  // (the first pass resets the solve's status, scales and weights)
   const double* b = rhs;
   if (out == rhs) {
     FDI_CUDA_TRY(cudaMemcpyAsync(p->ws[4], rhs, f.P * sizeof(double), cudaMemcpyDeviceToDevice, s));
@@ -1165,14 +1174,6 @@ fdi_status mixed_field_solve(fdi_plan* p, int field, double sigma, double lambda
   if (rblocks > p->npartials) {
     set_error("grid too large for the reduction buffer");
     return FDI_ERR_INVALID_ARG;
-  }
-  // flux weights multiplied by lambda for this solve
-  {
-    FDI_KTIMER(p, "reduce", s);
-    k_scale_weights<<<p->cyl ? 10 : 9, 256, 0, s>>>(mx->wp, mx->wm, mx->w0, nx, my->wp, my->wm, my->w0, ny, mz->wp,
-                                                    mz->wm, mz->w0, nz, p->cyl_wres_df, nz, split_host(lambda),
-                                                    p->lam_w);
-    FDI_LAUNCH_CHECK(p);
   }
   ResidArgs ra{};
   ra.nx = nx;
@@ -1214,10 +1215,27 @@ fdi_status mixed_field_solve(fdi_plan* p, int field, double sigma, double lambda
     a0.want_mean = singular ? 1 : 0;
     a0.rmax = p->d_scales + 0;
     a0.fin = FinishArgs{p->d_counter, p->partials, p->d_status, p->tol, 0, singular ? 1 : 0};
+    a0.fin.max_out = p->d_scales;
+    SetupArgs w{};
+    for (int d = 0; d < 3; ++d) {
+      const MixedAxis* m = static_cast<const MixedAxis*>(f.ax[d]->mixed);
+      const float2* src[3] = {m->wp, m->wm, m->w0};
+      for (int q = 0; q < 3; ++q) {
+        w.src[3 * d + q] = src[q];
+        w.n[3 * d + q] = f.n[d];
+      }
+    }
+    w.src[9] = p->cyl_wres_df;
+    w.n[9] = p->cyl ? nz : 0;
+    w.lambda = split_host(lambda);
+    w.lam_w = p->lam_w;
+    w.scales = p->d_scales;
+    w.nscales = (kMaxRefineCap + 2) * kScaleStride;
+    // the solve's first kernel: an ordinary launch
     if (px == nx && !singular && (reinterpret_cast<uintptr_t>(b) & 15u) == 0)
-      FDI_CUDA_TRY(launch_pdl(true, k_init_rhs_flat, dim3(fblocks), dim3(256), 0, s, a0, f.P));
+      FDI_CUDA_TRY(launch_pdl(false, k_init_rhs_flat, dim3(fblocks), dim3(256), 0, s, a0, w, f.P));
     else  // one warp per x-line: no more blocks than lines / 8
-      FDI_CUDA_TRY(launch_pdl(true, k_init_rhs, dim3(std::min(iblocks, (ny * nz + 7) / 8)), dim3(256), 0, s, a0));
+      FDI_CUDA_TRY(launch_pdl(false, k_init_rhs, dim3(std::min(iblocks, (ny * nz + 7) / 8)), dim3(256), 0, s, a0, w));
     FDI_LAUNCH_CHECK(p);
   }
 

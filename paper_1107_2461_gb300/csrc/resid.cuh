@@ -22,6 +22,8 @@ struct FinishArgs {
   // captured solves: condition of the next refinement round's graph node
   // (set to "not converged"); 0 when running eagerly
   cudaGraphConditionalHandle next_round = 0;
+  // kind 0: where the maximum of the records' first component (max |b|) goes
+  float* max_out = nullptr;
 };
 
 struct ResidArgs {

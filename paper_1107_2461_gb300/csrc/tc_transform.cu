@@ -145,79 +145,113 @@ __global__ void __launch_bounds__(THREADS, 1)
     tc::tmem_relinquish();
   }
   // per output column: the matrix row's scale (plan data), times the input's
-  // inverse scale below (both powers of two)
+  // inverse scale below (both powers of two); one column per epilogue thread
   float* s_cs = reinterpret_cast<float*>(smem + BAR_OFF + BAR_BYTES);
-  float csk[(NMAX + THREADS - 1) / THREADS];
-#pragma unroll
-  for (int q = 0; q < (NMAX + THREADS - 1) / THREADS; ++q) {
-    const int k = threadIdx.x + q * THREADS;
-    csk[q] = k < N_pad ? a.col_scale[k] : 0.f;
-  }
-  tc::tc_fence_before();
-  __syncthreads();
-  tc::tc_fence_after();
-  const uint32_t tmem_base = *tmem_slot;
-  // Everything above touches no data of the previous kernel in the stream, so
-  // under programmatic dependent launch it overlaps that kernel's tail; from
-  // here on the previous kernel has completed and its writes are visible.
-  pdl_wait();
-  const int skip = a.skip ? *a.skip : 0;  // the same for every thread
-  const float in_scale = a.scale_in ? *a.scale_in : 1.0f;
-  if (skip) {
-    if (warp == 1) tc::tmem_dealloc(tmem_base, tmem_cols);
-    return;
-  }
-  {
-    const float inv_s = 1.0f / scale_from_max(in_scale);
-#pragma unroll
-    for (int q = 0; q < (NMAX + THREADS - 1) / THREADS; ++q) {
-      const int k = threadIdx.x + q * THREADS;
-      if (k < N_pad) s_cs[k] = csk[q] * inv_s;
-    }
-  }
-  __syncthreads();
+  static_assert(NEPI * 32 == NMAX, "one column per epilogue thread");
+  const int ecol = threadIdx.x - (2 + NCONV) * 32;
+  const float csk = ecol >= 0 && ecol < N_pad ? a.col_scale[ecol] : 0.f;
 
-  const long long num_tiles = (a.R + BM - 1) / BM;
+  const int num_tiles = (int)((a.R + BM - 1) / BM);
   // work items: tiles below n_full whole, the tail's tiles as two halves
   // (columns [0, N_pad / 2) and [N_pad / 2, N_pad)); every role walks the same
   // items in the same order
-  const long long n_full = (a.n_full > 0 && a.n_full < num_tiles) ? a.n_full : num_tiles;
-  const long long num_items = n_full + 2 * (num_tiles - n_full);
-  const long long my_iters = blockIdx.x < num_items ? (num_items - 1 - blockIdx.x) / gridDim.x + 1 : 0;
+  const int n_full = (a.n_full > 0 && a.n_full < num_tiles) ? (int)a.n_full : num_tiles;
+  const int num_items = n_full + 2 * (num_tiles - n_full);
+  const int my_iters = (int)blockIdx.x < num_items ? (num_items - 1 - (int)blockIdx.x) / (int)gridDim.x + 1 : 0;
   // item `it` of this CTA: its tile, and half = -1 (whole), 0 or 1
-  auto item_tile = [&](long long it, int* half) -> long long {
-    const long long item = blockIdx.x + it * gridDim.x;
+  auto item_tile = [&](int it, int* half) -> int {
+    const int item = (int)blockIdx.x + it * (int)gridDim.x;
     if (item < n_full) {
       *half = -1;
       return item;
     }
-    const long long h = item - n_full;
-    *half = (int)(h & 1);
+    const int h = item - n_full;
+    *half = h & 1;
     return n_full + (h >> 1);
   };
   const int nK = a.nK;
+  const uint32_t total = (uint32_t)my_iters * (uint32_t)nK;
+  const uint32_t bbytes = (uint32_t)(2 * N_pad * ROWB);
+  auto load_b = [&](uint32_t g, int kc) {
+    const int s = g % NB;
+    tc::mbar_expect_tx(&full_b[s], bbytes);
+    tc::bulk_load(tc::smem_u32(smem + s * 2 * B_BYTES), a.img + (size_t)kc * bbytes, bbytes, &full_b[s]);
+  };
+  auto load_a = [&](uint32_t g, int it, int kc) {
+    int half = -1;
+    const int row0 = item_tile(it, &half) * BM;
+    const int sa = g % NA32;
+    const uint32_t dst = tc::smem_u32(smem + A32_OFF + sa * A32_BYTES);
+    tc::mbar_expect_tx(&a_full[sa], (uint32_t)A32_BYTES);
+    if (!a.a_mn) {
+      tc::tma_load_2d(dst, &tmA, kc * BK, row0, &a_full[sa]);
+    } else {
+      // MN-major input: box of 128 consecutive m (one slab) x 32 k rows
+      const int slab = row0 / (int)a.a_mslab;
+      tc::tma_load_2d(dst, &tmA, row0 - slab * (int)a.a_mslab, slab * a.K + kc * BK, &a_full[sa]);
+    }
+  };
+  tc::tc_fence_before();
+  __syncthreads();
+  tc::tc_fence_after();
+  const uint32_t tmem_base = *tmem_slot;
+  // The first chunks are requested as soon as they may be: the matrix (plan
+  // data) before the wait for the previous kernel, the input right after it,
+  // both without waiting for the skip flag and the scale (a round trip of 600
+  // clocks on a 64^3 pass of 8000).  Everything above and the matrix loads touch
+  // no data of the previous kernel in the stream, so under programmatic
+  // dependent launch they overlap that kernel's tail; after pdl_wait the
+  // previous kernel has completed and its writes are visible.
+  const uint32_t pre_b = total < NB ? total : NB, pre_a = total < NA32 ? total : NA32;
+  if (warp == 0 && lane == 0) {
+    int kc = 0;
+    for (uint32_t g = 0; g < pre_b; ++g) {
+      load_b(g, kc);
+      if (++kc == nK) kc = 0;
+    }
+  }
+  pdl_wait();
+  if (warp == WARP_A && lane == 0) {
+    int it = 0, kc = 0;
+    for (uint32_t g = 0; g < pre_a; ++g) {
+      load_a(g, it, kc);
+      if (++kc == nK) {
+        kc = 0;
+        ++it;
+      }
+    }
+  }
+  const int skip = a.skip ? *a.skip : 0;  // the same for every thread
+  const float in_scale = a.scale_in ? *a.scale_in : 1.0f;
+  if (skip) {
+    // the copies above still write shared memory
+    if (warp == 0 && lane == 0)
+      for (uint32_t g = 0; g < pre_b; ++g) tc::mbar_drain(&full_b[g], 0);
+    if (warp == WARP_A && lane == 0)
+      for (uint32_t g = 0; g < pre_a; ++g) tc::mbar_drain(&a_full[g], 0);
+    if (warp == 1) tc::tmem_dealloc(tmem_base, tmem_cols);
+    return;
+  }
 
   if (warp == 0) {
     // ---------------- producer of the B chunks (one bulk copy each) ----------------
     if (lane == 0) {
-      const uint32_t bbytes = (uint32_t)(2 * N_pad * ROWB);
       uint32_t g = 0;
-      for (long long it = 0; it < my_iters && !s_abort; ++it) {
+      for (int it = 0; it < my_iters && !s_abort; ++it) {
         for (int kc = 0; kc < nK; ++kc, ++g) {
-          const int s = g % NB;
-          const uint32_t ph = (g / NB) & 1;
-          if (!tc::mbar_wait(&empty_b[s], ph ^ 1, &s_abort, wl)) {
+          if (g < pre_b) continue;
+          if (!tc::mbar_wait(&empty_b[g % NB], ((g / NB) & 1) ^ 1, &s_abort, wl)) {
             s_abort = 1;
             atomicExch(a.err, 1);
             break;
           }
-          tc::mbar_expect_tx(&full_b[s], bbytes);
-          tc::bulk_load(tc::smem_u32(smem + s * 2 * B_BYTES), a.img + (size_t)kc * bbytes, bbytes, &full_b[s]);
+          load_b(g, kc);
         }
       }
       // the last NB loads issued may still be writing shared memory (after
       // a failure nobody consumes them); their phases complete regardless, and
       // a consumed one has completed already
+      if (g < pre_b) g = pre_b;
       for (uint32_t g2 = g > NB ? g - NB : 0; g2 < g; ++g2) tc::mbar_drain(&full_b[g2 % NB], (g2 / NB) & 1);
     }
   } else if (warp == 1) {
@@ -226,7 +260,7 @@ __global__ void __launch_bounds__(THREADS, 1)
     // vector registers, 166 instead of 128 clocks per 128 x 256 x 16 MMA)
     if (tc::elect_one()) {
       uint32_t g = 0;
-      for (long long it = 0; it < my_iters && !s_abort; ++it) {
+      for (int it = 0; it < my_iters && !s_abort; ++it) {
         int half = -1;
         item_tile(it, &half);
         // a half item accumulates its columns where the whole tile would
@@ -291,10 +325,8 @@ __global__ void __launch_bounds__(THREADS, 1)
     // k groups 0 .. 3
     const bool a_mn = a.a_mn != 0;
     const int c8 = ct & 3, r4 = ct >> 2;
-    const long long total = my_iters * nK;
     int kc = grp % nK;
-    for (long long gi = grp; gi < total && !s_abort; gi += 2) {
-      const uint32_t g = (uint32_t)gi;
+    for (uint32_t g = grp; g < total && !s_abort; g += 2) {
       const int sa = g % NA32, s = g % NS;
       if (!tc::mbar_wait(&a_full[sa], (g / NA32) & 1, &s_abort, wl)) {
         atomicExch(a.err, 4);
@@ -363,29 +395,18 @@ __global__ void __launch_bounds__(THREADS, 1)
     // ---------------- TMA producer (FP32 A) ----------------
     if (lane == 0) {
       uint32_t g = 0;
-      for (long long it = 0; it < my_iters && !s_abort; ++it) {
-        int half = -1;
-        const long long tile = item_tile(it, &half);
-        const int row0 = (int)(tile * BM);
+      for (int it = 0; it < my_iters && !s_abort; ++it) {
         for (int kc = 0; kc < nK; ++kc, ++g) {
-          const int sa = g % NA32;
-          const uint32_t pa = (g / NA32) & 1;
-          if (!tc::mbar_wait(&a_empty[sa], pa ^ 1, &s_abort, wl)) {
+          if (g < pre_a) continue;
+          if (!tc::mbar_wait(&a_empty[g % NA32], ((g / NA32) & 1) ^ 1, &s_abort, wl)) {
             s_abort = 1;
             atomicExch(a.err, 6);
             break;
           }
-          tc::mbar_expect_tx(&a_full[sa], (uint32_t)A32_BYTES);
-          if (!a.a_mn) {
-            tc::tma_load_2d(tc::smem_u32(smem + A32_OFF + sa * A32_BYTES), &tmA, kc * BK, row0, &a_full[sa]);
-          } else {
-            // MN-major input: box of 128 consecutive m (one slab) x 32 k rows
-            const long long slab = (long long)row0 / a.a_mslab;
-            tc::tma_load_2d(tc::smem_u32(smem + A32_OFF + sa * A32_BYTES), &tmA, (int)((long long)row0 % a.a_mslab),
-                            (int)(slab * a.K + (long long)kc * BK), &a_full[sa]);
-          }
+          load_a(g, it, kc);
         }
       }
+      if (g < pre_a) g = pre_a;
       for (uint32_t g2 = g > NA32 ? g - NA32 : 0; g2 < g; ++g2)
         tc::mbar_drain(&a_full[g2 % NA32], (g2 / NA32) & 1);
     }
@@ -400,6 +421,8 @@ __global__ void __launch_bounds__(THREADS, 1)
     // outputs) and stores them with one 16-byte access where the layout allows.
     const int q = warp & 3;  // TMEM lane quarter accessible to this warp
     const int ew = warp - (2 + NCONV), eh = ew >> 2;
+    if (ecol < N_pad) s_cs[ecol] = csk * (1.0f / scale_from_max(in_scale));
+    asm volatile("bar.sync 1, %0;" ::"n"(NEPI * 32) : "memory");
     float* tp = reinterpret_cast<float*>(smem + EPI_OFF + ew * EPI_WARP_BYTES);
     const bool rowmajor = a.col_stride == 1;
     // vector stores need 16-byte aligned groups of 4 along the contiguous index
@@ -409,9 +432,9 @@ __global__ void __launch_bounds__(THREADS, 1)
                        (reinterpret_cast<uintptr_t>(a.out_f32) & 15u) == 0;
     const int g8 = lane >> 3, l8 = lane & 7;  // after the transpose: group of 8 lanes, lane in group
     float vmax = 0.f;
-    for (long long it = 0; it < my_iters && !s_abort; ++it) {
+    for (int it = 0; it < my_iters && !s_abort; ++it) {
       int half = -1;
-      const long long tile = item_tile(it, &half);
+      const int tile = item_tile(it, &half);
       const int c_lo = half == 1 ? N_pad / 2 : 0, c_hi = half == 0 ? N_pad / 2 : N_pad;
       const int buf = (int)(it & 1);
       const uint32_t aph = (uint32_t)((it >> 1) & 1);
@@ -420,7 +443,7 @@ __global__ void __launch_bounds__(THREADS, 1)
         break;
       }
       tc::tc_fence_after();
-      const long long wrow0 = tile * BM + 32 * q;  // first row of this warp
+      const long long wrow0 = (long long)tile * BM + 32 * q;  // first row of this warp
       const bool tvalid = tile < num_tiles;
       const int nrows = tvalid ? (int)max(0LL, min((long long)32, a.R - wrow0)) : 0;
       // output base of this lane's own row (row = wrow0 + lane)
@@ -604,12 +627,14 @@ __global__ void __launch_bounds__(THREADS, 1)
       __syncwarp();
       if (lane == 0) tc::mbar_arrive(&acce[buf]);
     }
-    if (a.tma_store && lane == 0) tc::bulk_wait_all();
     if (a.scale_out) {
 #pragma unroll
       for (int o = 16; o > 0; o >>= 1) vmax = fmaxf(vmax, __shfl_xor_sync(0xffffffffu, vmax, o));
       if (lane == 0 && vmax > 0.f) atomicMax(reinterpret_cast<unsigned int*>(a.scale_out), __float_as_uint(vmax));
     }
+    // the stores must have read shared memory before the CTA gives it back (the
+    // grid completes after their writes)
+    if (a.tma_store && lane == 0) tc::bulk_wait_read_all();
   }
 
   tc::tc_fence_before();
