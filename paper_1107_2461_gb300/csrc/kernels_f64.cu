@@ -136,10 +136,86 @@ __device__ __forceinline__ void warp_max_out(float v, float* fmax) {
   if ((threadIdx.x & 31) == 0 && v > 0.f) atomicMax(reinterpret_cast<unsigned int*>(fmax), __float_as_uint(v));
 }
 
+// kTP planes per block of loads: every sweep reads its next block before it
+// computes the current one, so a step does not wait for memory (between events,
+// 64^3: 41 us with one step's loads in flight, 24 us in blocks of 8 or 16; 128^3:
+// 136, 57 and 47 us).  Single-warp blocks take 16; large fields keep 8, whose
+// registers leave enough warps per SM to stream 40 bytes per point (256^3 solve
+// 1.95 ms before, 1.82 with 8, 1.90 with 16).
+
+// The singular line of the zero-flux Laplacian (Eq. 28 reading), by a block of
+// its own: project the right-hand side to zero M_z-weighted mean, pin u_0 = 0,
+// solve rows 1 .. nz-1, remove the weighted mean of the solution.  The line is
+// staged in shared memory; the sums and copies run over the block's threads, the
+// recurrences in one.
 template <typename T>
+__device__ void thomas_singular_line(const ThomasArgs& a, const double* s_m, const double* s_lo, const T* in, T* out,
+                                     bool cached, float& vmax) {
+  __shared__ double s_f[kMaxN], s_c[kMaxN], s_i[kMaxN];
+  __shared__ double s_sum[2];
+  const int nz = a.nz, t = threadIdx.x;
+  for (int k = t; k < nz; k += blockDim.x) {
+    s_f[k] = (double)in[k * a.kstride];
+    if (cached) {
+      s_i[k] = a.cinv[k * a.q];
+      s_c[k] = a.ccp[k * a.q];
+    }
+  }
+  __syncthreads();
+  auto weighted = [&]() {  // (sum M, sum M s_f) by the first warp
+    if (t < 32) {
+      double sm = 0.0, sf = 0.0;
+      for (int k = t; k < nz; k += 32) {
+        sm += s_m[k];
+        sf = fma(s_m[k], s_f[k], sf);
+      }
+      const double v = red::warp_sum2(sm, sf);
+      if (t == 0) s_sum[0] = v;
+      if (t == 16) s_sum[1] = v;
+    }
+    __syncthreads();
+    return s_sum[1] / s_sum[0];
+  };
+  const double mu = weighted();
+  if (t == 0) {
+    double cprev = 0.0, dprev = 0.0;
+    for (int k = 1; k < nz; ++k) {
+      const double lo = (k > 1) ? -s_lo[k - 1] : 0.0;
+      double inv;
+      if (cached) {
+        inv = s_i[k];
+      } else {
+        const double up = (k + 1 < nz) ? -s_lo[k] : 0.0;
+        inv = 1.0 / (-a.lambda * a.kdz[k] - lo * cprev);
+        cprev = up * inv;
+        s_i[k] = inv;
+        s_c[k] = cprev;
+      }
+      dprev = (s_m[k] * (s_f[k] - mu) - lo * dprev) * inv;
+      s_f[k] = dprev;
+    }
+    double u = dprev;
+    for (int k = nz - 2; k >= 1; --k) {
+      u = s_f[k] - s_c[k] * u;
+      s_f[k] = u;
+    }
+    s_f[0] = 0.0;
+  }
+  __syncthreads();
+  const double mean = weighted();
+  for (int k = t; k < nz; k += blockDim.x) {
+    const double w = s_f[k] - mean;
+    out[k * a.kstride] = (T)w;
+    vmax = fmaxf(vmax, fabsf((float)w));
+    if (a.cinv && !cached) {
+      a.cinv[k * a.q] = s_i[k];
+      a.ccp[k * a.q] = s_c[k];
+    }
+  }
+}
+
+template <typename T, int kTP>
 __global__ void __launch_bounds__(128) k_thomas_f64(ThomasArgs a, const int* __restrict__ skip) {
-  pdl_wait();
-  if (skip && *skip) return;
   __shared__ double s_m[kMaxN], s_lo[kMaxN];  // M_k and lambda K_{k,k+1}
   const int nz = a.nz;
   for (int k = threadIdx.x; k < nz; k += blockDim.x) {
@@ -147,13 +223,15 @@ __global__ void __launch_bounds__(128) k_thomas_f64(ThomasArgs a, const int* __r
     s_lo[k] = a.lambda * a.koz[k];
   }
   __syncthreads();
+  pdl_wait();  // (the coefficients are plan data)
+  if (skip && *skip) return;
   const long long NL = (long long)a.nx * a.ny;
+  // a singular problem has one block more, which solves the null line (0, 0)
+  const bool null_block = a.singular_possible && blockIdx.x == gridDim.x - 1;
   const long long l0 = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   float vmax = 0.f;
-  // lines past the end run line NL - 1 again without storing (the warp stays
-  // whole for the max reduction)
-  const bool live = l0 < NL;
-  const long long l = live ? l0 : NL - 1;
+  const long long l = null_block ? 0 : (l0 < NL ? l0 : NL - 1);
+  const bool live = !null_block && l0 < NL && !(a.singular_possible && l0 == 0);
   int i, j;
   long long off;
   if (a.mixed_layout) {
@@ -168,92 +246,101 @@ __global__ void __launch_bounds__(128) k_thomas_f64(ThomasArgs a, const int* __r
   const T* in = static_cast<const T*>(a.in) + off;
   T* out = static_cast<T*>(a.out) + off;
   const long long ks = a.kstride;
-  const double lab = a.lamx[i] + a.lamy[j];
-  // the y eigenvalue takes its own weight on cylindrical plans (Eq. 44: the
-  // theta eigenvalue multiplies the discrete 1/r^2 of the radial cell)
-  const double s = a.sigma - a.lambda * (a.wy ? a.lamx[i] : lab);
-  const double ly = a.wy ? a.lambda * a.lamy[j] : 0.0;
-  const double lam = a.lambda;
-  if (!(a.singular_possible && lab == 0.0)) {
-    const bool cached = a.cinv && a.key[0] == a.sigma && a.key[1] == a.lambda && a.key[2] == (double)a.field;
+  const bool cached = a.cinv && a.key[0] == a.sigma && a.key[1] == a.lambda && a.key[2] == (double)a.field;
+  if (null_block) {
+    thomas_singular_line<T>(a, s_m, s_lo, in, out, cached, vmax);
+  } else if (live) {
+    const double lab = a.lamx[i] + a.lamy[j];
+    // the y eigenvalue takes its own weight on cylindrical plans (Eq. 44: the
+    // theta eigenvalue multiplies the discrete 1/r^2 of the radial cell)
+    const double s = a.sigma - a.lambda * (a.wy ? a.lamx[i] : lab);
+    const double ly = a.wy ? a.lambda * a.lamy[j] : 0.0;
+    const double lam = a.lambda;
     double* cp_arr = a.cinv ? a.ccp + l : a.cs + off;
     const long long cstride = a.cinv ? a.q : ks;
-    if (cached && live) {
-      const double* inv = a.cinv + l;
-      double d = 0.0;
-      for (int k = 0; k < nz; ++k) {
-        double t = __dmul_rn(s_m[k], (double)in[k * ks]);
-        if (k > 0) t = __fma_rn(s_lo[k - 1], d, t);
-        d = __dmul_rn(t, inv[k * a.q]);
-        out[k * ks] = (T)d;
+    const double* inv_arr = a.cinv + l;
+    T f[kTP], fn[kTP];
+    double iv[kTP], ivn[kTP];
+    auto load_fwd = [&](int k0, T (&x)[kTP], double (&y)[kTP]) {
+#pragma unroll
+      for (int u = 0; u < kTP; ++u) {
+        const int k = min(k0 + u, nz - 1);
+        x[u] = in[k * ks];
+        if (cached) y[u] = inv_arr[k * a.q];
       }
-      double u = d;
-      vmax = fmaxf(vmax, fabsf((float)u));
-      for (int k = nz - 2; k >= 0; --k) {
-        u = __fma_rn(-cp_arr[k * cstride], u, (double)out[k * ks]);
-        out[k * ks] = (T)u;
-        vmax = fmaxf(vmax, fabsf((float)u));
+    };
+    double d = 0.0;
+    load_fwd(0, f, iv);
+    if (cached) {
+      for (int k0 = 0; k0 < nz; k0 += kTP) {
+        if (k0 + kTP < nz) load_fwd(k0 + kTP, fn, ivn);
+#pragma unroll
+        for (int u = 0; u < kTP; ++u) {
+          const int k = k0 + u;
+          if (k < nz) {
+            double t = __dmul_rn(s_m[k], (double)f[u]);
+            if (k > 0) t = __fma_rn(s_lo[k - 1], d, t);
+            d = __dmul_rn(t, iv[u]);
+            out[k * ks] = (T)d;
+          }
+          f[u] = fn[u];
+          iv[u] = ivn[u];
+        }
       }
-    } else if (live) {
-      double cprev = 0.0, dprev = 0.0;
-      for (int k = 0; k < nz; ++k) {
-        const double lo = (k > 0) ? -s_lo[k - 1] : 0.0;
-        const double up = (k + 1 < nz) ? -s_lo[k] : 0.0;
-        double di = s * s_m[k] - lam * a.kdz[k];
-        if (a.wy) di -= ly * a.wy[k];
-        const double inv = 1.0 / (di - lo * cprev);
-        cprev = up * inv;
-        // the same operations, in the same order, as the cached sweep: a
-        // solve gives the same bits whether its factors were cached or not
-        double t = __dmul_rn(s_m[k], (double)in[k * ks]);
-        if (k > 0) t = __fma_rn(s_lo[k - 1], dprev, t);
-        dprev = __dmul_rn(t, inv);
-        cp_arr[k * cstride] = cprev;
-        if (a.cinv) a.cinv[l + k * a.q] = inv;
-        out[k * ks] = (T)dprev;
-      }
-      double u = dprev;
-      vmax = fmaxf(vmax, fabsf((float)u));
-      for (int k = nz - 2; k >= 0; --k) {
-        u = __fma_rn(-cp_arr[k * cstride], u, (double)out[k * ks]);
-        out[k * ks] = (T)u;
-        vmax = fmaxf(vmax, fabsf((float)u));
+    } else {
+      double cprev = 0.0;
+      for (int k0 = 0; k0 < nz; k0 += kTP) {
+        if (k0 + kTP < nz) load_fwd(k0 + kTP, fn, ivn);
+#pragma unroll 1
+        for (int u = 0; u < kTP; ++u) {
+          const int k = k0 + u;
+          if (k >= nz) break;
+          const double lo = (k > 0) ? -s_lo[k - 1] : 0.0;
+          const double up = (k + 1 < nz) ? -s_lo[k] : 0.0;
+          double di = s * s_m[k] - lam * a.kdz[k];
+          if (a.wy) di -= ly * a.wy[k];
+          const double inv = 1.0 / (di - lo * cprev);
+          cprev = up * inv;
+          // the same operations, in the same order, as the cached sweep: a
+          // solve gives the same bits whether its factors were cached or not
+          double t = __dmul_rn(s_m[k], (double)f[0]);
+          if (k > 0) t = __fma_rn(s_lo[k - 1], d, t);
+          d = __dmul_rn(t, inv);
+          cp_arr[k * cstride] = cprev;
+          if (a.cinv) a.cinv[l + k * a.q] = inv;
+          out[k * ks] = (T)d;
+#pragma unroll
+          for (int q = 0; q + 1 < kTP; ++q) f[q] = f[q + 1];
+        }
+#pragma unroll
+        for (int u = 0; u < kTP; ++u) f[u] = fn[u];
       }
     }
-  } else if (live) {
-    // singular line of the zero-flux Laplacian (Eq. 28 reading): project the
-    // right-hand side to zero M_z-weighted mean, pin u_0 = 0, solve rows 1..nz-1,
-    // then remove the weighted mean of the solution.
-    double* cs = a.cs + off;
-    double sm = 0.0, sf = 0.0;
-    for (int k = 0; k < nz; ++k) {
-      sm += s_m[k];
-      sf += s_m[k] * (double)in[k * ks];
-    }
-    const double mu = sf / sm;
-    double cprev = 0.0, dprev = 0.0;
-    for (int k = 1; k < nz; ++k) {
-      const double lo = (k > 1) ? -s_lo[k - 1] : 0.0;
-      const double up = (k + 1 < nz) ? -s_lo[k] : 0.0;
-      const double di = s * s_m[k] - lam * a.kdz[k];
-      const double inv = 1.0 / (di - lo * cprev);
-      cprev = up * inv;
-      dprev = (s_m[k] * ((double)in[k * ks] - mu) - lo * dprev) * inv;
-      cs[k * ks] = cprev;
-      out[k * ks] = (T)dprev;
-    }
-    double u = dprev, su = s_m[nz - 1] * dprev;
-    for (int k = nz - 2; k >= 1; --k) {
-      u = (double)out[k * ks] - cs[k * ks] * u;
-      out[k * ks] = (T)u;
-      su += s_m[k] * u;
-    }
-    out[0] = (T)0.0;
-    const double mean = su / sm;
-    for (int k = 0; k < nz; ++k) {
-      const double w = (double)out[k * ks] - mean;
-      out[k * ks] = (T)w;
-      vmax = fmaxf(vmax, fabsf((float)w));
+    // back substitution, blocks from the top: f holds d', iv holds c'
+    auto load_back = [&](int k0, T (&x)[kTP], double (&y)[kTP]) {
+#pragma unroll
+      for (int u = 0; u < kTP; ++u) {
+        const int k = max(k0 - u, 0);
+        x[u] = out[k * ks];
+        y[u] = cp_arr[k * cstride];
+      }
+    };
+    double u_ = d;
+    vmax = fmaxf(vmax, fabsf((float)u_));
+    load_back(nz - 2, f, iv);
+    for (int k0 = nz - 2; k0 >= 0; k0 -= kTP) {
+      if (k0 - kTP >= 0) load_back(k0 - kTP, fn, ivn);
+#pragma unroll
+      for (int u = 0; u < kTP; ++u) {
+        const int k = k0 - u;
+        if (k >= 0) {
+          u_ = __fma_rn(-iv[u], u_, (double)f[u]);
+          out[k * ks] = (T)u_;
+          vmax = fmaxf(vmax, fabsf((float)u_));
+        }
+        f[u] = fn[u];
+        iv[u] = ivn[u];
+      }
     }
   }
   // one reduction point for the whole warp
@@ -273,6 +360,9 @@ __global__ void __launch_bounds__(128) k_thomas_f64(ThomasArgs a, const int* __r
     }
   }
 }
+
+// threads per block: single warps while that still leaves SM quarters idle
+int thomas_threads(long long lines) { return lines <= 152 * 128 ? 32 : 128; }
 
 __global__ void k_divide_f64(double* __restrict__ data, int nx, int ny, int nz, const double* __restrict__ lx,
                              const double* __restrict__ ly, const double* __restrict__ lz, double sigma,
@@ -615,7 +705,9 @@ fdi_status launch_thomas_f64(fdi_plan* p, const Field& f, double sigma, double l
     a.key = p->tf + 2 * p->tf_q;
     a.ticket = p->d_counter + 1;
   }
-  FDI_CUDA_TRY(launch_pdl(p->pdl, k_thomas_f64<double>, dim3((unsigned)((NL + 127) / 128)), dim3(128), 0, s, a, skip));
+  const int nt = thomas_threads(NL);
+  FDI_CUDA_TRY(launch_pdl(p->pdl, nt == 32 ? k_thomas_f64<double, 16> : k_thomas_f64<double, 8>, dim3((unsigned)((NL + nt - 1) / nt) + a.singular_possible),
+                          dim3(nt), 0, s, a, skip));
   FDI_LAUNCH_CHECK(p);
   return FDI_OK;
 }
@@ -650,7 +742,11 @@ fdi_status launch_thomas_cached_f32(fdi_plan* p, const Field& f, double sigma, d
   a.ccp = p->tf + p->tf_q;
   a.key = p->tf + 2 * p->tf_q;
   a.ticket = p->d_counter + 1;
-  k_thomas_f64<float><<<(unsigned)((NL + 127) / 128), 128, 0, s>>>(a, skip);
+  const int nt = thomas_threads(NL);
+  if (nt == 32)
+    k_thomas_f64<float, 16><<<(unsigned)((NL + nt - 1) / nt), nt, 0, s>>>(a, skip);
+  else
+    k_thomas_f64<float, 8><<<(unsigned)((NL + nt - 1) / nt), nt, 0, s>>>(a, skip);
   FDI_LAUNCH_CHECK(p);
   return FDI_OK;
 }
