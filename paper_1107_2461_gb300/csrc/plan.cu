@@ -393,9 +393,12 @@ fdi_status finish_plan(fdi_plan* p, cudaStream_t s) {
     // digit planes of the transformed directions (z only for the Cartesian TPF)
     FDI_TRY(dev_alloc(&p->d_err, 1));
     FDI_CUDA_TRY(cudaMemsetAsync(p->d_err, 0, sizeof(int), s));
-    const int nd = (p->thomas_axis == -1 && !p->cyl) ? 3 : 2;
-    for (int fi = 0; fi < p->nfields; ++fi)
-      for (int d = 0; d < nd; ++d) FDI_TRY(slice_prepare_axis(p, p->fields[fi].ax[d], s));
+    const bool tz = p->thomas_axis == -1 && !p->cyl;
+    for (int fi = 0; fi < p->nfields; ++fi) {
+      const Field& f = p->fields[fi];
+      for (int d = 0; d < 2 && !small_plane_f64(f); ++d) FDI_TRY(slice_prepare_axis(p, f.ax[d], s));
+      if (tz && !small_z_f64(f)) FDI_TRY(slice_prepare_axis(p, f.ax[2], s));
+    }
     FDI_CUDA_TRY(cudaStreamSynchronize(s));
     FDI_CUDA_TRY(cudaStreamCreateWithFlags(&p->cstream, cudaStreamNonBlocking));
   }

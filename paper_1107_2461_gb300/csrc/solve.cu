@@ -20,6 +20,7 @@
 
 #include "fdi_internal.h"
 #include "resident.h"
+#include "slice_transform.h"
 
 namespace fdi {
 
@@ -91,33 +92,45 @@ fdi_status solve_once_f64(fdi_plan* p, int field, double sigma, double lambda, c
   double* t0 = p->ws[0];
   double* t1 = p->ws[1];
   double* t2 = p->ws[2];
+  const bool small = small_plane_f64(f);
   auto fwd = [&](int d, const double* src, double* dst) {
     return launch_axis_f64(p, f, d, true, src, dst, false, d > 0, skip, s);
   };
   auto back = [&](int d, const double* src, double* dst, bool acc) {
     return launch_axis_f64(p, f, d, false, src, dst, acc, true, skip, s);
   };
-  FDI_TRY(fwd(0, in, t0));
-  FDI_TRY(fwd(1, t0, t1));
+  // in -> t1 in the x and y eigenbases
+  if (small) {
+    FDI_TRY(launch_small_plane(p, f, true, in, t1, false, false, skip, s));
+  } else {
+    FDI_TRY(fwd(0, in, t0));
+    FDI_TRY(fwd(1, t0, t1));
+  }
+  // t1 -> z
+  double* z = t0;
   if (p->thomas_axis == 2) {
     FDI_TRY(launch_thomas_f64(p, f, sigma, lambda, field, t1, t0, t2, skip, s));
-    FDI_TRY(back(1, t0, t1, false));
-    FDI_TRY(back(0, t1, out, accumulate));
   } else if (p->cyl) {
     // cylindrical TPF (Eq. 45-46): the radial transform of theta mode j uses
     // that mode's own eigenbasis, the divide its own eigenvalues
     FDI_TRY(launch_modes_f64(p, t1, t0, p->cyl_Eri, nz, nx, ny, skip, s));
     FDI_TRY(launch_divide_modes_f64(p, f, sigma, lambda, t0, skip, s));
     FDI_TRY(launch_modes_f64(p, t0, t1, p->cyl_Er, nz, nx, ny, skip, s));
-    FDI_TRY(back(1, t1, t0, false));
-    FDI_TRY(back(0, t0, out, accumulate));
+    z = t1;
+  } else if (small_z_f64(f)) {
+    FDI_TRY(launch_small_z(p, f, sigma, lambda, t1, skip, s));
+    z = t1;
   } else {
     FDI_TRY(fwd(2, t1, t0));
     FDI_TRY(launch_divide_f64(p, f, sigma, lambda, t0, skip, s));
     FDI_TRY(back(2, t0, t1, false));
-    FDI_TRY(back(1, t1, t0, false));
-    FDI_TRY(back(0, t0, out, accumulate));
+    z = t1;
   }
+  // z -> out
+  if (small) return launch_small_plane(p, f, false, z, out, accumulate, true, skip, s);
+  double* y = z == t0 ? t1 : t0;
+  FDI_TRY(back(1, z, y, false));
+  FDI_TRY(back(0, y, out, accumulate));
   return FDI_OK;
 }
 

@@ -1,5 +1,6 @@
-"""FP64 eigenvector transforms (digit products on the tensor cores) at the edges
-of their tiles: 16-column steps, 128-mode tiles, 32 and 64 lines per item.
+"""FP64 eigenvector transforms (digit products on the tensor cores, plain FP64 on
+small planes) at the edges of their tiles: 16-column steps, 128-mode tiles, 32 and
+64 lines per item, planes of up to 32 x 32 cells.
 
 With lambda = 0 the operator is the identity, so a solve is the forward and
 back transforms alone: u must equal f.  z-planes do not mix then, and each one
@@ -37,7 +38,9 @@ def solve(fdi, plan, lam, f):
 
 
 @pytest.mark.parametrize("n", [(2, 3, 5), (15, 16, 6), (17, 33, 5), (31, 64, 5), (65, 63, 9), (127, 129, 5),
-                               (128, 130, 60), (40, 200, 61), (255, 256, 5), (256, 241, 5)])
+                               (128, 130, 60), (40, 200, 61), (255, 256, 5), (256, 241, 5),
+                               # both plane transforms (and the z steps) in one launch up to 32 cells
+                               (32, 32, 32), (32, 31, 33), (33, 32, 32), (3, 30, 17)])
 @pytest.mark.parametrize("axis", [2, -1])
 def test_transforms_invert_each_other(fdi, n, axis):
     faces = [tanh_faces(n[d], 1.5) for d in range(3)]
