@@ -90,41 +90,84 @@ __device__ __forceinline__ df::F2 ld2(const float2* p) {
 constexpr int kResTX = 32, kResTY = 8, kResZChunk = 16;  // planes per block (at most)
 constexpr int kResBX = 2 * kResTX;                       // x columns per block
 
-struct Acc {
-  float h, l;  // unnormalised double-float accumulator
+// Both points of a pair run through the same operations, two FP32 values per
+// instruction (f32x2: the same roundings as the scalar forms, half the issue
+// slots, which bound the exact body: 209 thread instructions per point at 80%
+// issue with scalar arithmetic: 124 us at 256^3, 118 us packed, when the FP32 pipe,
+// which still takes a clock per value, is what is left; whole solve 546 to 537 us).
+struct V2 {
+  unsigned long long u;
 };
 
-__device__ __forceinline__ void acc_add(Acc& s, float ph, float pl) {
-  const float t = s.h + ph;
-  const float bb = t - s.h;
-  s.l += ((s.h - (t - bb)) + (ph - bb)) + pl;
+__device__ __forceinline__ V2 v2(float a, float b) {
+  V2 r;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(r.u) : "f"(a), "f"(b));
+  return r;
+}
+__device__ __forceinline__ void unpack(V2 v, float& a, float& b) {
+  asm("mov.b64 {%0, %1}, %2;" : "=f"(a), "=f"(b) : "l"(v.u));
+}
+__device__ __forceinline__ V2 add2(V2 a, V2 b) {
+  V2 r;
+  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r.u) : "l"(a.u), "l"(b.u));
+  return r;
+}
+__device__ __forceinline__ V2 mul2(V2 a, V2 b) {
+  V2 r;
+  asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r.u) : "l"(a.u), "l"(b.u));
+  return r;
+}
+__device__ __forceinline__ V2 fma2(V2 a, V2 b, V2 c) {
+  V2 r;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r.u) : "l"(a.u), "l"(b.u), "l"(c.u));
+  return r;
+}
+__device__ __forceinline__ V2 minus1() { return V2{0xbf800000bf800000ull}; }
+// a - b as one rounding of a + (-1) b
+__device__ __forceinline__ V2 sub2(V2 a, V2 b) { return fma2(b, minus1(), a); }
+
+struct Acc {
+  V2 h, l;  // unnormalised double-float accumulators of the two points
+};
+
+// s += p, given (p exact in its high part) the low part q (or none)
+template <bool LOW>
+__device__ __forceinline__ void acc_add(Acc& s, V2 p, V2 q) {
+  const V2 t = add2(s.h, p);
+  const V2 bb = sub2(t, s.h);
+  V2 e = add2(sub2(s.h, sub2(t, bb)), sub2(p, bb));
+  if (LOW) e = add2(e, q);
+  s.l = add2(s.l, e);
   s.h = t;
 }
 
 // a - c = d + dl exactly (Knuth two-difference)
 struct Diff {
-  float d, dl;
+  V2 d, dl;
 };
 
-__device__ __forceinline__ Diff two_diff(float a, float c) {
-  const float d = a - c;
-  const float bb = d - a;
-  return Diff{d, (a - (d - bb)) - (c + bb)};
+__device__ __forceinline__ Diff two_diff(V2 a, V2 c) {
+  const V2 d = sub2(a, c);
+  const V2 bb = sub2(d, a);
+  return Diff{d, sub2(sub2(a, sub2(d, bb)), add2(c, bb))};
 }
 
-__device__ __forceinline__ Diff neg(Diff t) { return Diff{-t.d, -t.dl}; }
+// high and low parts of a double-float weight for the two points
+struct W2 {
+  V2 x, y;
+};
 
 // s += w * (d + dl) for a double-float weight w: the high product enters by
 // two-sum, its exact rounding error and the two small cross products by FMA
 // into the low part
-__device__ __forceinline__ void acc_flux(Acc& s, float2 w, Diff t) {
-  const float p = w.x * t.d;
-  const float e = fmaf(w.x, t.d, -p);
-  const float tt = s.h + p;
-  const float bb = tt - s.h;
-  float l = fmaf(w.x, t.dl, s.l);
-  l = fmaf(w.y, t.d, l);
-  s.l = l + (((s.h - (tt - bb)) + (p - bb)) + e);
+__device__ __forceinline__ void acc_flux(Acc& s, W2 w, Diff t) {
+  const V2 p = mul2(w.x, t.d);
+  const V2 e = fma2(w.x, t.d, mul2(p, minus1()));
+  const V2 tt = add2(s.h, p);
+  const V2 bb = sub2(tt, s.h);
+  V2 l = fma2(w.x, t.dl, s.l);
+  l = fma2(w.y, t.d, l);
+  s.l = add2(l, add2(add2(sub2(s.h, sub2(tt, bb)), sub2(p, bb)), e));
   s.h = tt;
 }
 
@@ -132,56 +175,45 @@ __device__ __forceinline__ void acc_flux(Acc& s, float2 w, Diff t) {
 // first residual is small (FAST): the difference rounded once, the flux
 // product added by FMA to the high part, other terms added in FP32.
 template <bool FAST>
-__device__ __forceinline__ Diff diff_of(float a, float c) {
-  if (FAST) return Diff{a - c, 0.f};
+__device__ __forceinline__ Diff diff_of(V2 a, V2 c) {
+  if (FAST) return Diff{sub2(a, c), V2{0ull}};
   return two_diff(a, c);
 }
 
 template <bool FAST>
-__device__ __forceinline__ void flux_of(Acc& s, float2 w, Diff t) {
+__device__ __forceinline__ void flux_of(Acc& s, W2 w, Diff t) {
   if (FAST)
-    s.h = fmaf(w.x, t.d, s.h);
+    s.h = fma2(w.x, t.d, s.h);
   else
     acc_flux(s, w, t);
 }
 
-template <bool FAST>
-__device__ __forceinline__ void add_of(Acc& s, float ph, float pl) {
+template <bool FAST, bool LOW>
+__device__ __forceinline__ void add_of(Acc& s, V2 p, V2 q) {
   if (FAST) {
-    s.h += ph;
-    s.l += pl;
+    s.h = add2(s.h, p);
+    if (LOW) s.l = add2(s.l, q);
   } else {
-    acc_add(s, ph, pl);
+    acc_add<LOW>(s, p, q);
   }
 }
 
 // one x pair of FP32 values (hi) and, for LO, of the low plane
 struct Pair {
-  float a, b;     // points i0, i0 + 1
-  float la, lb;   // low parts (LO only)
+  V2 v, l;
 };
 
 template <bool VEC, bool LO>
 __device__ __forceinline__ Pair ld_pair(const float* hi, const float* lo, int o, int d1) {
-  Pair v{0.f, 0.f, 0.f, 0.f};
+  Pair r{V2{0ull}, V2{0ull}};
   if (VEC) {
-    const float2 h = *reinterpret_cast<const float2*>(hi + o);
-    v.a = h.x;
-    v.b = h.y;
-    if (LO) {
-      const float2 l = *reinterpret_cast<const float2*>(lo + o);
-      v.la = l.x;
-      v.lb = l.y;
-    }
+    r.v.u = *reinterpret_cast<const unsigned long long*>(hi + o);
+    if (LO) r.l.u = *reinterpret_cast<const unsigned long long*>(lo + o);
   } else {
-    v.a = hi[o];
-    v.b = hi[o + d1];
-    if (LO) {
-      v.la = lo[o];
-      v.lb = lo[o + d1];
-    }
+    r.v = v2(hi[o], hi[o + d1]);
+    if (LO) r.l = v2(lo[o], lo[o + d1]);
   }
-  return v;
+  return r;
 }
 
 // Two residual passes share this body.
@@ -223,12 +255,14 @@ __device__ __forceinline__ void resid_body(const ResidArgs& a, double* sh, int b
     mean_l = -mb.lo;
   }
   const int ib = ia + d1;
-  const float2 wpxa = a.wp[0][ia], wmxa = a.wm[0][ia], wpxb = a.wp[0][ib], wmxb = a.wm[0][ib];
-  float2 wpy = make_float2(0.f, 0.f), wmy = wpy;
+  auto both = [](float2 p, float2 q) { return W2{v2(p.x, q.x), v2(p.y, q.y)}; };
+  const W2 wpx = both(a.wp[0][ia], a.wp[0][ib]), wmx = both(a.wm[0][ia], a.wm[0][ib]);
+  W2 wpy{}, wmy{};
   float2 w0y = make_float2(0.f, 0.f);
   if (!CYL) {
-    wpy = a.wp[1][jc];
-    wmy = a.wm[1][jc];
+    const float2 p = a.wp[1][jc], m = a.wm[1][jc];
+    wpy = both(p, p);
+    wmy = both(m, m);
     w0y = a.w0[1][jc];
   }
   const float2 w0xa = a.w0[0][ia], w0xb = a.w0[0][ib];
@@ -283,9 +317,7 @@ __device__ __forceinline__ void resid_body(const ResidArgs& a, double* sh, int b
   };
   auto ldr1 = [&](int o, Pair& q) { q = ld_pair<VEC, true>(q1h, q1l, o, d1); };
   auto ldh = [&](int o, float& h0, float& h1) {
-    const Pair q = ld_pair<VEC, false>(hc, nullptr, o, d1);
-    h0 = q.a;
-    h1 = q.b;
+    unpack(ld_pair<VEC, false>(hc, nullptr, o, d1).v, h0, h1);
   };
   // pipeline: pair C at plane k and P at k + 1, rows below (S) and above (N)
   // and the edge value E at plane k, and the right-hand side parts of plane k
@@ -297,21 +329,20 @@ __device__ __forceinline__ void resid_body(const ResidArgs& a, double* sh, int b
   float El = 0.f;
   float E = lde(ok, El);
   double b0 = 0.0, b1 = 0.0;
-  Pair Q{0.f, 0.f, 0.f, 0.f};
+  Pair Q{V2{0ull}, V2{0ull}};
   float h0 = 0.f, h1 = 0.f;
   if (MODE == 0) ldb(ok, b0, b1);
   if (MODE == 1) ldr1(rk, Q);
   if (MODE == 1 && (OUT || MEAN)) ldh(ok, h0, h1);
-  // exact z differences of the faces below plane k (u_{k-1} - u_k) and the
-  // low parts of plane k-1 (LO); at k = 0 the clamped plane gives zero
-  Diff dza, dzb;
-  float mla = 0.f, mlb = 0.f;
+  // z differences across the faces below plane k (u_k - u_{k-1}; the flux takes
+  // the negated weight) and the low parts of plane k-1 (LO); at k = 0 the
+  // clamped plane gives zero
+  Diff dz;
+  V2 ml{0ull};
   {
     const Pair M = ldp(uhc, ulc, max(k0 - 1, 0) * szi);
-    dza = diff_of<FAST>(M.a, C.a);
-    dzb = diff_of<FAST>(M.b, C.b);
-    mla = M.la;
-    mlb = M.lb;
+    dz = diff_of<FAST>(C.v, M.v);
+    ml = M.l;
   }
   const float2* wpz = a.wp[2];
   const float2* wmz = a.wm[2];
@@ -338,41 +369,39 @@ __device__ __forceinline__ void resid_body(const ResidArgs& a, double* sh, int b
       if (MODE == 1 && (OUT || MEAN)) ldh(o1, h02, h12);
     }
     // x neighbours outside the pair: from the neighbouring lanes, or the edge value
-    const float sd = __shfl_down_sync(0xffffffffu, C.a, 1);
-    const float su = __shfl_up_sync(0xffffffffu, C.b, 1);
-    const float eb = lane == kResTX - 1 ? E : sd;   // east of point b
-    const float wa = lane == 0 ? E : su;            // west of point a
-    float ebl = 0.f, wal = 0.f;
+    float ca, cb, cla = 0.f, clb = 0.f;
+    unpack(C.v, ca, cb);
+    const float sd = __shfl_down_sync(0xffffffffu, ca, 1);
+    const float su = __shfl_up_sync(0xffffffffu, cb, 1);
+    const V2 east = v2(cb, lane == kResTX - 1 ? E : sd);
+    const V2 west = v2(lane == 0 ? E : su, ca);
+    V2 eastl{0ull}, westl{0ull};
     if (MODE == 1 && LO) {
-      const float sdl = __shfl_down_sync(0xffffffffu, C.la, 1);
-      const float sul = __shfl_up_sync(0xffffffffu, C.lb, 1);
-      ebl = lane == kResTX - 1 ? El : sdl;
-      wal = lane == 0 ? El : sul;
+      unpack(C.l, cla, clb);
+      const float sdl = __shfl_down_sync(0xffffffffu, cla, 1);
+      const float sul = __shfl_up_sync(0xffffffffu, clb, 1);
+      eastl = v2(clb, lane == kResTX - 1 ? El : sdl);
+      westl = v2(lane == 0 ? El : sul, cla);
     }
-    Acc Sa, Sb;
+    Acc A;
     df::F2 ba = df::make(0.f, 0.f), bb = ba;
     if (MODE == 0) {
       ba = df::from_f64(b0);
       bb = df::from_f64(b1);
-      Sa = Acc{ba.hi, ba.lo};
-      Sb = Acc{bb.hi, bb.lo};
-      if (MEAN) {
-        add_of<FAST>(Sa, mean_h, mean_l);
-        add_of<FAST>(Sb, mean_h, mean_l);
-      }
+      A = Acc{v2(ba.hi, bb.hi), v2(ba.lo, bb.lo)};
+      if (MEAN) add_of<FAST, true>(A, v2(mean_h, mean_h), v2(mean_l, mean_l));
     } else {
-      Sa = Acc{Q.a, Q.la};
-      Sb = Acc{Q.b, Q.lb};
+      A = Acc{Q.v, Q.l};
     }
     if (MEAN) {
       const df::F2 mz = ld2(a.m[2] + k);
       const df::F2 Vka = df::mul(Va, mz), Vkb = df::mul(Vb, mz);
-      df::F2 xa = df::make(C.a, 0.f), xb = df::make(C.b, 0.f);
+      df::F2 xa = df::make(ca, 0.f), xb = df::make(cb, 0.f);
       if (MODE == 1) {
-        xa = df::two_sum(h0, C.a);
-        xa = df::fast_two_sum(xa.hi, xa.lo + C.la);
-        xb = df::two_sum(h1, C.b);
-        xb = df::fast_two_sum(xb.hi, xb.lo + C.lb);
+        xa = df::two_sum(h0, ca);
+        xa = df::fast_two_sum(xa.hi, xa.lo + cla);
+        xb = df::two_sum(h1, cb);
+        xb = df::fast_two_sum(xb.hi, xb.lo + clb);
       }
       if (act0) {
         svb = df::add(svb, df::mul(Vka, xa));
@@ -384,70 +413,64 @@ __device__ __forceinline__ void resid_body(const ResidArgs& a, double* sh, int b
       }
     }
     const float2 wpzk = wpz[k], wmzk = wmz[k];
+    const float2 nwmz = make_float2(-wmzk.x, -wmzk.y);
     if (CYL) {
-      wpy = a.wy[k];
+      const float2 w = a.wy[k];
+      wpy = both(w, w);
       wmy = wpy;
     }
-    // point a: east (the pair's inner face), west, south, north, up, down
-    const Diff dab = diff_of<FAST>(C.b, C.a);
-    const Diff dua = diff_of<FAST>(P.a, C.a), dub = diff_of<FAST>(P.b, C.b);
-    flux_of<FAST>(Sa, wpxa, dab);
-    flux_of<FAST>(Sa, wmxa, diff_of<FAST>(wa, C.a));
-    flux_of<FAST>(Sa, wmy, diff_of<FAST>(S.a, C.a));
-    flux_of<FAST>(Sa, wpy, diff_of<FAST>(N.a, C.a));
-    flux_of<FAST>(Sa, wpzk, dua);
-    flux_of<FAST>(Sa, wmzk, dza);
-    // point b
-    flux_of<FAST>(Sb, wpxb, diff_of<FAST>(eb, C.b));
-    flux_of<FAST>(Sb, wmxb, neg(dab));
-    flux_of<FAST>(Sb, wmy, diff_of<FAST>(S.b, C.b));
-    flux_of<FAST>(Sb, wpy, diff_of<FAST>(N.b, C.b));
-    flux_of<FAST>(Sb, wpzk, dub);
-    flux_of<FAST>(Sb, wmzk, dzb);
-    float sla = 0.f, slb = 0.f;  // lambda L applied to the low parts, FP32
+    // east, west, south, north, up, down
+    flux_of<FAST>(A, wpx, diff_of<FAST>(east, C.v));
+    flux_of<FAST>(A, wmx, diff_of<FAST>(west, C.v));
+    flux_of<FAST>(A, wmy, diff_of<FAST>(S.v, C.v));
+    flux_of<FAST>(A, wpy, diff_of<FAST>(N.v, C.v));
+    const Diff du = diff_of<FAST>(P.v, C.v);
+    flux_of<FAST>(A, both(wpzk, wpzk), du);
+    flux_of<FAST>(A, both(nwmz, nwmz), dz);
+    V2 sl{0ull};  // lambda L applied to the low parts, FP32
     if (MODE == 1 && LO) {
-      sla = fmaf(wpxa.x, C.lb - C.la, sla);
-      sla = fmaf(wmxa.x, wal - C.la, sla);
-      sla = fmaf(wmy.x, S.la - C.la, sla);
-      sla = fmaf(wpy.x, N.la - C.la, sla);
-      sla = fmaf(wpzk.x, P.la - C.la, sla);
-      sla = fmaf(wmzk.x, mla - C.la, sla);
-      slb = fmaf(wpxb.x, ebl - C.lb, slb);
-      slb = fmaf(wmxb.x, C.la - C.lb, slb);
-      slb = fmaf(wmy.x, S.lb - C.lb, slb);
-      slb = fmaf(wpy.x, N.lb - C.lb, slb);
-      slb = fmaf(wpzk.x, P.lb - C.lb, slb);
-      slb = fmaf(wmzk.x, mlb - C.lb, slb);
+      sl = fma2(wpx.x, sub2(eastl, C.l), sl);
+      sl = fma2(wmx.x, sub2(westl, C.l), sl);
+      sl = fma2(wmy.x, sub2(S.l, C.l), sl);
+      sl = fma2(wpy.x, sub2(N.l, C.l), sl);
+      sl = fma2(v2(wpzk.x, wpzk.x), sub2(P.l, C.l), sl);
+      sl = fma2(v2(wmzk.x, wmzk.x), sub2(ml, C.l), sl);
     }
     const float2 w0k = w0z[k];
     if (wall_xy || w0k.x != 0.f) {  // wall term: only next to a Dirichlet wall
       const df::F2 wyz = df::add(df::make(w0y.x, w0y.y), df::make(w0k.x, w0k.y));
-      const df::F2 ta = df::mul(df::add(df::make(w0xa.x, w0xa.y), wyz), df::make(C.a, C.la));
-      const df::F2 tb = df::mul(df::add(df::make(w0xb.x, w0xb.y), wyz), df::make(C.b, C.lb));
-      add_of<FAST>(Sa, ta.hi, ta.lo);
-      add_of<FAST>(Sb, tb.hi, tb.lo);
+      const df::F2 ta = df::mul(df::add(df::make(w0xa.x, w0xa.y), wyz), df::make(ca, cla));
+      const df::F2 tb = df::mul(df::add(df::make(w0xb.x, w0xb.y), wyz), df::make(cb, clb));
+      add_of<FAST, true>(A, v2(ta.hi, tb.hi), v2(ta.lo, tb.lo));
     }
     if (SIG == 1) {
-      add_of<FAST>(Sa, -C.a, -C.la);
-      add_of<FAST>(Sb, -C.b, -C.lb);
+      add_of<FAST, (MODE == 1 && LO)>(A, mul2(C.v, minus1()), mul2(C.l, minus1()));
     } else if (SIG == 2) {
       const df::F2 sg = df::make(a.sigma.x, a.sigma.y);
-      const df::F2 ta = df::mul(sg, df::make(C.a, C.la));
-      const df::F2 tb = df::mul(sg, df::make(C.b, C.lb));
-      add_of<FAST>(Sa, -ta.hi, -ta.lo);
-      add_of<FAST>(Sb, -tb.hi, -tb.lo);
+      const df::F2 ta = df::mul(sg, df::make(ca, cla));
+      const df::F2 tb = df::mul(sg, df::make(cb, clb));
+      add_of<FAST, true>(A, v2(-ta.hi, -tb.hi), v2(-ta.lo, -tb.lo));
     }
-    // S.h + S.l: the rounding errors in S.l may exceed the cancelled S.h, so
-    // the pair is rounded with a full two-sum
-    const df::F2 ra = FAST ? df::make(Sa.h + (Sa.l + sla), 0.f) : df::two_sum(Sa.h, Sa.l + sla);
-    const df::F2 rb = FAST ? df::make(Sb.h + (Sb.l + slb), 0.f) : df::two_sum(Sb.h, Sb.l + slb);
+    // h + l: the rounding errors in l may exceed the cancelled h, so the pair is
+    // rounded with a full two-sum
+    df::F2 ra, rb;
+    {
+      const V2 lsum = (MODE == 1 && LO) ? add2(A.l, sl) : A.l;
+      const V2 t = add2(A.h, lsum);
+      unpack(t, ra.hi, rb.hi);
+      ra.lo = rb.lo = 0.f;
+      if (!FAST) {
+        const V2 q = sub2(t, A.h);
+        unpack(add2(sub2(A.h, sub2(t, q)), sub2(lsum, q)), ra.lo, rb.lo);
+      }
+    }
     // stores: the pair at once where both points exist
     {
       double oa = 0.0, ob = 0.0;
       if (OUT) {
         // every lane of the warp runs this (f2d_warp votes)
-        oa = df::f2d_warp(h0) + (LO ? df::f2d_warp(C.a) + df::f2d_warp(C.la) : df::f2d_warp(C.a));
-        ob = df::f2d_warp(h1) + (LO ? df::f2d_warp(C.b) + df::f2d_warp(C.lb) : df::f2d_warp(C.b));
+        oa = df::f2d_warp(h0) + (LO ? df::f2d_warp(ca) + df::f2d_warp(cla) : df::f2d_warp(ca));
+        ob = df::f2d_warp(h1) + (LO ? df::f2d_warp(cb) + df::f2d_warp(clb) : df::f2d_warp(cb));
       }
       if (VEC && act0) {  // VEC: act0 implies act1
         *reinterpret_cast<float2*>(rc + rk) = make_float2(ra.hi, rb.hi);
@@ -476,10 +499,8 @@ __device__ __forceinline__ void resid_body(const ResidArgs& a, double* sh, int b
       if (MODE == 0) sbb = MEAN ? fmaf(bb.hi + mean_h, bb.hi + mean_h, sbb) : fmaf(bb.hi, bb.hi, sbb);
       rmax = fmaxf(rmax, fabsf(rb.hi));
     }
-    dza = neg(dua);
-    dzb = neg(dub);
-    mla = C.la;
-    mlb = C.lb;
+    dz = du;
+    ml = C.l;
     C = P;
     P = P2;
     S = S2;
