@@ -523,11 +523,90 @@ __device__ __forceinline__ void cp_async8(unsigned dst, const float2* src) {
   asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"(dst), "l"(src) : "memory");
 }
 
+// The pair of lines that holds the singular line of the zero-flux Laplacian,
+// (0, 0) and (0, 1), in a block of its own: the pair is staged in shared memory
+// by the whole block, thread 0 projects, pins and re-centres the null line,
+// thread 1 sweeps its neighbour, with the arithmetic of k_thomas_f32 (so the
+// same values).  It runs beside the other blocks of the sweep: as a launch of
+// its own after them, working on global memory, it held up every round of a
+// Laplace solve (a 128^3 projection step of three Helmholtz solves and one
+// Laplace solve went from 762 to 579 us, a 64^3 Stokes solve, whose
+// preconditioner has one Laplace solve per iteration, from 5.78 to 5.41 ms).
+// Cartesian plans only (a cylindrical zero-flux Laplacian is refused).  Returns
+// the largest magnitude this thread wrote.  buf: 4 * kMaxN floats of shared memory
+__device__ float thomas_null_pair(const Thomas32Args& a, const float4* co, float* buf) {
+  const int nz = a.nz, tid = threadIdx.x;
+  const bool second = a.ny > 1;
+  float* fv = buf;               // [line][nz]
+  float* cv = buf + 2 * kMaxN;   // [line][nz]: c'
+  for (int e = tid; e < 2 * nz; e += blockDim.x) {
+    const int l = e & 1, k = e >> 1;
+    if (l == 0 || second) fv[l * kMaxN + k] = a.f[k * a.plane + l];
+  }
+  __syncthreads();
+  if (tid == 0) {
+    const float s = (float)(a.sigma - a.lambda * (a.lamx[0] + a.lamy[0]));
+    float sm = 0.f, sf = 0.f;
+    for (int k = 0; k < nz; ++k) {
+      sm += co[k].x;
+      sf = fmaf(co[k].x, fv[k], sf);
+    }
+    const float mu = sf / sm;
+    float cp = 0.f, dp = 0.f;
+    for (int k = 1; k < nz; ++k) {
+      const float4 c = co[k];
+      thomas_step(s, c.x, c.y, k > 1 ? c.z : 0.f, c.w, fv[k] - mu, cp, dp);
+      cv[k] = cp;
+      fv[k] = dp;
+    }
+    float u = dp, su = co[nz - 1].x * dp;
+    for (int k = nz - 2; k >= 1; --k) {
+      u = fmaf(-cv[k], u, fv[k]);
+      fv[k] = u;
+      su = fmaf(co[k].x, u, su);
+    }
+    fv[0] = 0.f;
+    const float mean = su / sm;
+    for (int k = 0; k < nz; ++k) fv[k] -= mean;
+  } else if (tid == 1 && second) {
+    const float s = (float)(a.sigma - a.lambda * (a.lamx[0] + a.lamy[1]));
+    float* f1 = fv + kMaxN;
+    float* c1 = cv + kMaxN;
+    float cp = 0.f, dp = 0.f;
+    for (int k = 0; k < nz; ++k) {
+      const float4 c = co[k];
+      const float inv = rcp_fast(fmaf(-c.z, cp, thomas_diag<false>(s, 0.f, c, nullptr, k)));
+      cp = c.w * inv;
+      dp = fmaf(c.x, f1[k], -c.z * dp) * inv;
+      c1[k] = cp;
+      f1[k] = dp;
+    }
+    float u = 0.f;
+    for (int k = nz - 1; k >= 0; --k) {
+      u = fmaf(-c1[k], u, f1[k]);
+      f1[k] = u;
+    }
+  }
+  __syncthreads();
+  float vmax = 0.f;
+  for (int e = tid; e < 2 * nz; e += blockDim.x) {
+    const int l = e & 1, k = e >> 1;
+    if (l == 0 || second) {
+      const float w = fv[l * kMaxN + k];
+      a.f[k * a.plane + l] = w;
+      vmax = fmaxf(vmax, fabsf(w));
+    }
+  }
+  return vmax;
+}
+
 // FP32 Thomas sweep, two adjacent lines (i, j) and (i, j + 1) per thread (j
 // even): the copies, shared-memory reads, stores and coefficient reads are
 // shared by the two recurrences, which also give the thread two independent
-// dependency chains.  A pair holding the singular line of the zero-flux
-// Laplacian is left to k_thomas_f32 (launched over that pair only).  When ny
+// dependency chains.  The pair holding the singular line of the zero-flux
+// Laplacian is left to thomas_null_pair, in block 0 of a grid that has one
+// block more for it (SING; its own instances, since the code beside the sweep made
+// other solves 0.4 to 1.6% slower, 16^3 78.7 -> 80.0 us).  When ny
 // is odd the last pair's second line is a padding column of the row: it is
 // swept with a valid eigenvalue and excluded from the scale.
 // The forward elimination stores nothing but c' and d' at the block
@@ -538,7 +617,7 @@ __device__ __forceinline__ void cp_async8(unsigned dst, const float2* src) {
 // bytes) instead of f read, d' written and read back, u written (16 bytes);
 // the top kNBR blocks are still in the copy ring when the back substitution
 // starts and are not read again.
-template <int TL, bool FULL, bool CYL>
+template <int TL, bool FULL, bool CYL, bool SING>
 __global__ void __launch_bounds__(TL) k_thomas2_f32(Thomas32Args a, const int* __restrict__ skip) {
   pdl_wait();
   if (skip && *skip) return;
@@ -558,15 +637,17 @@ __global__ void __launch_bounds__(TL) k_thomas2_f32(Thomas32Args a, const int* _
   __syncthreads();
   const int tid = threadIdx.x;
   const int npair = (a.ny + 1) / 2;
-  const long long t = (long long)blockIdx.x * blockDim.x + tid;
+  const long long t = (long long)((int)blockIdx.x - (SING ? 1 : 0)) * blockDim.x + tid;
   float vmax = 0.f;
-  if (t < (long long)a.nx * npair) {
+  if (SING && t < 0) {
+    vmax = thomas_null_pair(a, s_co, reinterpret_cast<float*>(&ring[0][0]));
+  } else if (t < (long long)a.nx * npair) {
     const int i = (int)(t / npair), j0 = 2 * (int)(t % npair);
     const bool second = j0 + 1 < a.ny;
     const int pl2 = (int)(a.plane / 2);  // plane stride in float2 (plane and pitch are even)
     const double lab0 = a.lamx[i] + a.lamy[j0];
     const double lab1 = a.lamx[i] + a.lamy[second ? j0 + 1 : j0];
-    if (!(a.singular_possible && (lab0 == 0.0 || lab1 == 0.0))) {
+    if (!(SING && (lab0 == 0.0 || lab1 == 0.0))) {
       const float s0 = (float)(a.sigma - a.lambda * (CYL ? a.lamx[i] : lab0));
       const float s1 = (float)(a.sigma - a.lambda * (CYL ? a.lamx[i] : lab1));
       const float ly0 = CYL ? (float)(-a.lamy[j0]) : 0.f;
@@ -670,7 +751,7 @@ __global__ void __launch_bounds__(TL) k_thomas2_f32(Thomas32Args a, const int* _
 constexpr int kTopBlocks = 8;
 constexpr int kTopBytes = kTopBlocks * kTB * 64 * (int)sizeof(float2);
 
-template <bool FULL, bool CYL>
+template <bool FULL, bool CYL, bool SING>
 __global__ void __launch_bounds__(64) k_thomas2c_f32(Thomas32Args a, const int* __restrict__ skip) {
   constexpr int TL = 64;
   pdl_wait();
@@ -691,15 +772,17 @@ __global__ void __launch_bounds__(64) k_thomas2c_f32(Thomas32Args a, const int* 
   __syncthreads();
   const int tid = threadIdx.x;
   const int npair = (a.ny + 1) / 2;
-  const long long t = (long long)blockIdx.x * blockDim.x + tid;
+  const long long t = (long long)((int)blockIdx.x - (SING ? 1 : 0)) * blockDim.x + tid;
   float vmax = 0.f;
-  if (t < (long long)a.nx * npair) {
+  if (SING && t < 0) {
+    vmax = thomas_null_pair(a, s_co, reinterpret_cast<float*>(&ring[0][0]));
+  } else if (t < (long long)a.nx * npair) {
     const int i = (int)(t / npair), j0 = 2 * (int)(t % npair);
     const bool second = j0 + 1 < a.ny;
     const int pl2 = (int)(a.plane / 2);
     const double lab0 = a.lamx[i] + a.lamy[j0];
     const double lab1 = a.lamx[i] + a.lamy[second ? j0 + 1 : j0];
-    if (!(a.singular_possible && (lab0 == 0.0 || lab1 == 0.0))) {
+    if (!(SING && (lab0 == 0.0 || lab1 == 0.0))) {
       const float s0 = (float)(a.sigma - a.lambda * (CYL ? a.lamx[i] : lab0));
       const float s1 = (float)(a.sigma - a.lambda * (CYL ? a.lamx[i] : lab1));
       const float ly0 = CYL ? (float)(-a.lamy[j0]) : 0.f;
@@ -1061,55 +1144,25 @@ fdi_status resident_describe(fdi_plan* p, int field, double sigma, double lambda
 
 // FP32 Thomas sweep in the configuration of the plan (thomas_tl)
 template <bool CYL>
-fdi_status launch_thomas32(fdi_plan* p, const Thomas32Args& ta, bool pdl, bool singular, const int* skip,
-                           cudaStream_t s) {
+fdi_status launch_thomas32(fdi_plan* p, const Thomas32Args& ta, bool pdl, const int* skip, cudaStream_t s) {
   const long long lines = (long long)ta.nx * ta.ny;
   const bool full = ta.nz % kTB == 0;
-  if (p->thomas_tl == 2) {
-    // two lines per thread, 64 threads (128 lines) per CTA
+  if (p->thomas_tl == 2 || p->thomas_tl == 3) {
+    // two lines per thread, 64 threads (128 lines) per CTA; 3: with the top
+    // planes' d' on chip
+    const bool top = p->thomas_tl == 3, sing = !CYL && ta.singular_possible;
     const long long pairs = (long long)ta.nx * ((ta.ny + 1) / 2);
-    const unsigned g = (unsigned)((pairs + 63) / 64);
-    if (full)
-      FDI_CUDA_TRY(launch_pdl(pdl, k_thomas2_f32<64, true, CYL>, dim3(g), dim3(64), 0, s, ta, skip));
-    else
-      FDI_CUDA_TRY(launch_pdl(pdl, k_thomas2_f32<64, false, CYL>, dim3(g), dim3(64), 0, s, ta, skip));
+    const unsigned g = (unsigned)((pairs + 63) / 64) + (sing ? 1u : 0u);
+    using Kernel = void (*)(Thomas32Args, const int*);
+    constexpr bool S = !CYL;  // the singular instances exist for Cartesian plans only
+    const Kernel k2[2][2] = {{k_thomas2_f32<64, false, CYL, false>, k_thomas2_f32<64, false, CYL, S>},
+                             {k_thomas2_f32<64, true, CYL, false>, k_thomas2_f32<64, true, CYL, S>}};
+    const Kernel k2c[2][2] = {{k_thomas2c_f32<false, CYL, false>, k_thomas2c_f32<false, CYL, S>},
+                              {k_thomas2c_f32<true, CYL, false>, k_thomas2c_f32<true, CYL, S>}};
+    const Kernel k = (top ? k2c : k2)[full ? 1 : 0][sing ? 1 : 0];
+    if (top) FDI_CUDA_TRY(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, kTopBytes));
+    FDI_CUDA_TRY(launch_pdl(pdl, k, dim3(g), dim3(64), top ? (size_t)kTopBytes : 0, s, ta, skip));
     FDI_LAUNCH_CHECK(p);
-    if (singular) {
-      // the null line (0, 0) and its pair partner, one line per thread
-      Thomas32Args t1 = ta;
-      t1.nx = 1;
-      t1.ny = std::min(ta.ny, 2);
-      if (full)
-        k_thomas_f32<64, true, CYL><<<1, 64, 0, s>>>(t1, skip);
-      else
-        k_thomas_f32<64, false, CYL><<<1, 64, 0, s>>>(t1, skip);
-      FDI_LAUNCH_CHECK(p);
-    }
-    return FDI_OK;
-  }
-  if (p->thomas_tl == 3) {
-    // two lines per thread with the top planes' d' on chip
-    static bool attr[2] = {false, false};
-    auto kfull = k_thomas2c_f32<true, CYL>;
-    auto kpart = k_thomas2c_f32<false, CYL>;
-    if (!attr[full ? 1 : 0]) {
-      FDI_CUDA_TRY(cudaFuncSetAttribute(full ? kfull : kpart, cudaFuncAttributeMaxDynamicSharedMemorySize, kTopBytes));
-      attr[full ? 1 : 0] = true;
-    }
-    const long long pairs = (long long)ta.nx * ((ta.ny + 1) / 2);
-    const unsigned g = (unsigned)((pairs + 63) / 64);
-    FDI_CUDA_TRY(launch_pdl(pdl, full ? kfull : kpart, dim3(g), dim3(64), (size_t)kTopBytes, s, ta, skip));
-    FDI_LAUNCH_CHECK(p);
-    if (singular) {
-      Thomas32Args t1 = ta;
-      t1.nx = 1;
-      t1.ny = std::min(ta.ny, 2);
-      if (full)
-        k_thomas_f32<64, true, CYL><<<1, 64, 0, s>>>(t1, skip);
-      else
-        k_thomas_f32<64, false, CYL><<<1, 64, 0, s>>>(t1, skip);
-      FDI_LAUNCH_CHECK(p);
-    }
     return FDI_OK;
   }
   if (p->thomas_tl == 64) {
@@ -1357,9 +1410,9 @@ fdi_status mixed_field_solve(fdi_plan* p, int field, double sigma, double lambda
       if (p->thomas_tl == 4 && p->tf && !singular)
         FDI_TRY(launch_thomas_cached_f32(p, f, sigma, lambda, field, F2, py, (long long)nx * py, sc + 2, skip, s));
       else if (p->cyl)
-        FDI_TRY(launch_thomas32<true>(p, ta, pdl, singular, skip, s));
+        FDI_TRY(launch_thomas32<true>(p, ta, pdl, skip, s));
       else
-        FDI_TRY(launch_thomas32<false>(p, ta, pdl, singular, skip, s));
+        FDI_TRY(launch_thomas32<false>(p, ta, pdl, skip, s));
     }
     // back y: F2 [z][i][j] -> F4
     t.in = F2;
