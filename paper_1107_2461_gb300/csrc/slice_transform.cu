@@ -25,16 +25,19 @@
 // Layout: T is the MMA's A operand (M = 128 output modes), 64 grid lines are
 // its B operand (N = 64): eight FP32 accumulators of 64 columns fill tensor
 // memory, and a line is converted to digits only once per 128 modes.  Per
-// 16-column step of the contraction 36 MMAs (128 x 64 x 16) run from one stage
-// of 8 digit planes of T (32 KB, one bulk copy from L2) and 8 of the lines
-// (16 KB, written by the converters); consecutive products share the A operand,
-// which stays in the tensor core's collector buffer.
+// 16-column step of the contraction the 36 products run from one stage of 8 digit
+// planes of T (32 KB, one bulk copy from L2) and 8 of the lines (16 KB, written by
+// the converters).  The digit planes of the lines follow one another, so up to
+// four of them are one B operand of N = 256 rows, and its products with digit u of
+// T fall into the neighbouring accumulators of levels u + v, u + v + 1, ..: 12 MMAs
+// instead of 36 that each read the 4 KB of T again.
 //
 // Measured (GB300, x or y pass of a 256^3 field): 6.89 ms with FP64 multiply-adds,
-// 0.30 ms here;
-// a 128^3 field 0.29 -> 0.045 ms, 48 x 64 x 40 cells 27 -> 9 us.  The MMAs are
-// bound by shared-memory reads (104 KB of operands per step at 128 B/clk), about
-// 43 clocks each; the rest of an item (10 of 40 thousand clocks) is the epilogue.
+// 0.30 ms with one MMA per product, 0.27 ms here; a whole FP64 solve of 256^3
+// 28.6 -> 1.80 -> 1.70 ms, of 128^3 256 -> 248 us from the joined products.  Of the
+// 34 thousand clocks of an item (64 lines, 256 columns) the MMAs take 18 (bound by
+// their shared-memory reads, 120 KB per step at 128 B/clk), 11 are the epilogue,
+// which holds all of tensor memory, 5 waits for operands.
 //
 // Warp roles of the persistent CTA (one per SM, 704 threads):
 //   warp 0       bulk copies of the digit planes of T
@@ -108,27 +111,14 @@ __host__ __device__ __forceinline__ uint32_t sw32_offset(int row, int h) {
   return (uint32_t)(row * 32 + ((h ^ ((row >> 2) & 1)) << 4));
 }
 
-// one product of digit planes; REUSE: 0 the A operand is read and kept in the
-// collector buffer, 1 taken from there, 2 taken from there for the last time,
-// 3 read and not kept
-template <int REUSE>
+// digit planes of the lines times one digit plane of T
 __device__ __forceinline__ void mma_digits(uint32_t d, uint64_t a, uint64_t b, uint32_t idesc, uint32_t acc) {
-#define FDI_MMA_DIGITS(col)                                                                  \
-  asm volatile(                                                                              \
-      "{\n\t.reg .pred p;\n\t"                                                               \
-      "setp.ne.b32 p, %4, 0;\n\t"                                                            \
-      "tcgen05.mma.cta_group::1.kind::f16" col " [%0], %1, %2, %3, p;\n\t}" ::"r"(d),        \
-      "l"(a), "l"(b), "r"(idesc), "r"(acc)                                                   \
-      : "memory")
-  if (REUSE == 0)
-    FDI_MMA_DIGITS(".collector::a::fill");
-  else if (REUSE == 1)
-    FDI_MMA_DIGITS(".collector::a::use");
-  else if (REUSE == 2)
-    FDI_MMA_DIGITS(".collector::a::lastuse");
-  else
-    FDI_MMA_DIGITS("");
-#undef FDI_MMA_DIGITS
+  asm volatile(
+      "{\n\t.reg .pred p;\n\t"
+      "setp.ne.b32 p, %4, 0;\n\t"
+      "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}" ::"r"(d),
+      "l"(a), "l"(b), "r"(idesc), "r"(acc)
+      : "memory");
 }
 
 __device__ __forceinline__ void tmem_ld4(uint32_t taddr, float (&r)[4]) {
@@ -321,9 +311,9 @@ __global__ void __launch_bounds__(THREADS, 1) k_slice_transform(const SliceArgs 
         tc::mbar_drain(&full[g2 % STAGES], (g2 / STAGES) & 1);
     }
   } else if (warp == 1) {
-    // one elected thread (under a lane test 56-76 clocks per MMA instead of 35)
+    // one elected thread (under a lane test 56-76 clocks per N = 64 MMA instead of 35)
     if (tc::elect_one()) {
-      const uint32_t idesc = tc::idesc_f16_f32(TM, TN);
+      constexpr int NPL = 256 / TN;  // digit planes of the lines per MMA (N <= 256)
       const uint32_t s_base = tc::smem_u32(smem);
       uint32_t g = 0;
       for (int it = 0; it < items && !s_abort; ++it) {
@@ -343,23 +333,19 @@ __global__ void __launch_bounds__(THREADS, 1) k_slice_transform(const SliceArgs 
           tc::tc_fence_after();
           const uint32_t sa = s_base + s * SM::STAGE_BYTES, sb = sa + A_BYTES;
           // digit u of T times digit v of the lines goes to level u + v; the
-          // first step's u = 0 products start every level
+          // first step's u = 0 products start every level.  Up to 256 rows of
+          // the digit planes v, v + 1, .. are one B operand, whose products with
+          // digit u land in the neighbouring columns of levels u + v, u + v + 1, ..
 #pragma unroll
           for (int u = 0; u < SL; ++u) {
             const uint64_t da = sdesc_k_sw32(sa + u * A_SLICE);
             const uint32_t acc = (kc > 0 || u > 0) ? 1u : 0u;
 #pragma unroll
-            for (int v = 0; v < SL - u; ++v) {
+            for (int v = 0; v < SL - u; v += NPL) {
+              const int planes = SL - u - v < NPL ? SL - u - v : NPL;
               const uint32_t d = tmem + (uint32_t)((u + v) * TN);
               const uint64_t db = sdesc_k_sw32(sb + v * SM::B_SLICE);
-              if (u == SL - 1)
-                mma_digits<3>(d, da, db, idesc, acc);
-              else if (v == 0)
-                mma_digits<0>(d, da, db, idesc, acc);
-              else if (v == SL - u - 1)
-                mma_digits<2>(d, da, db, idesc, acc);
-              else
-                mma_digits<1>(d, da, db, idesc, acc);
+              mma_digits(d, da, db, tc::idesc_f16_f32(TM, planes * TN), acc);
             }
           }
           tc::mma_commit(&freed[(g + STAGES) % GROUPS]);
