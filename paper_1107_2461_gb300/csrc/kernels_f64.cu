@@ -816,11 +816,16 @@ fdi_status launch_residual_f64(fdi_plan* p, const Field& f, double sigma, double
   a.partials = p->partials;
   a.ticket = p->d_counter;
   a.next_round = next_round;
-  // short marches where longer ones leave SMs without a block (the extra plane
-  // differenced per march is 1/13 of a plane's operations)
+  // the march length with the least work on the busiest SM, a march costing its
+  // planes and about one plane's time for its start (a whole FP64 solve with 8, the
+  // longest, and with the rule's length: 64^3 86 and 78 us, 80^3 133 and 125, 112^3
+  // 214 and 209, 128^3 246 and 238; from 48^3 to 256^3 no other length was faster)
   const dim3 cols((unsigned)((a.nx + 63) / 64), (unsigned)((a.ny + 7) / 8));
+  auto blocks = [&](int zc) { return (long long)cols.x * cols.y * ((a.nz + zc - 1) / zc); };
+  auto cost = [&](int zc) { return (blocks(zc) + 151) / 152 * (zc + 1); };
   a.zchunk = kResZ;
-  while (a.zchunk > 1 && (long long)cols.x * cols.y * ((a.nz + a.zchunk - 1) / a.zchunk) < 304) a.zchunk /= 2;
+  for (int zc = kResZ - 1; zc >= 1; --zc)
+    if (cost(zc) < cost(a.zchunk) && blocks(zc) <= p->npartials) a.zchunk = zc;
   const dim3 grid(cols.x, cols.y, (unsigned)((a.nz + a.zchunk - 1) / a.zchunk));
   if ((long long)grid.x * grid.y * grid.z > p->npartials) {
     set_error("grid too large for the reduction buffer");
