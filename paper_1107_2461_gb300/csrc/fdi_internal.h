@@ -164,7 +164,7 @@ struct fdi_plan {
   // afterwards (a small LRU set, so alternating buffers keep their graphs)
   bool use_graphs = true;
   bool pdl = true;                  // programmatic dependent launch between a solve's kernels
-  bool loop_capture = false;        // capturing the body of the device-side Krylov loop
+  bool own_capture = false;         // capturing this plan's solve (or a batch with it) for the library's own graph
   // mixed field solves run one direct solve only (no residual check, no
   // refinement; FP64 output of the first solve): set around preconditioner
   // applications, which need no more than an approximate inverse

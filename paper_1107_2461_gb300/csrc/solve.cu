@@ -163,10 +163,12 @@ fdi_status field_solve_internal(fdi_plan* p, int field, double sigma, double lam
   // the one before it, so a converged solve launches nothing more (a 16^3 solve
   // went from 80 to 58 us with its residual's reduction folded in, 64^3 from 127
   // to 105 us).
-  // Inside the Krylov loop's WHILE body the rounds stay ordinary launches: there,
-  // with the solves joined from side streams right after their conditional
-  // nodes, a replay never finished (the GPU idle, the host waiting).
-  cudaGraph_t g = (p->max_refine >= 1 && !p->loop_capture) ? capturing_graph(s) : nullptr;
+  // Only in the graphs of field_solve_entry and batch_solve.  In a caller's own
+  // capture the rounds stay ordinary launches (a graph with conditional nodes
+  // cannot be used everywhere a plain one can), and in the Krylov loop's WHILE
+  // body too: there, with the solves joined from side streams right after their
+  // conditional nodes, a replay never finished (the GPU idle, the host waiting).
+  cudaGraph_t g = (p->max_refine >= 1 && p->own_capture) ? capturing_graph(s) : nullptr;
   if (!g) {
     for (int round = 0; round <= p->max_refine; ++round) FDI_TRY(enqueue_round(round, s, 0));
     return FDI_OK;
@@ -266,6 +268,17 @@ cudaStream_t capture_stream(fdi_plan* p, cudaStream_t s) {
   return p->gstream;
 }
 
+// marks plans whose launches go into one of the library's own graphs
+struct OwnCapture {
+  fdi_plan* const* plans;
+  int count;
+  OwnCapture(fdi_plan* const* q, int n) : plans(q), count(n) { set(true); }
+  ~OwnCapture() { set(false); }
+  void set(bool on) {
+    for (int i = 0; i < count; ++i) plans[i]->own_capture = on;
+  }
+};
+
 bool same_key(const fdi_plan::GraphKey& a, const fdi_plan::GraphKey& b) {
   return a.field == b.field && a.sigma == b.sigma && a.lambda == b.lambda && a.rhs == b.rhs && a.out == b.out &&
          a.s == b.s;
@@ -326,7 +339,11 @@ fdi_status field_solve_entry(fdi_plan* p, int field, double sigma, double lambda
   const cudaStream_t cs = capture_stream(p, s);
   if (!cs) return field_solve(p, field, sigma, lambda, rhs, out, s);
   FDI_CUDA_TRY(cudaStreamBeginCapture(cs, cudaStreamCaptureModeThreadLocal));
-  fdi_status st = field_solve(p, field, sigma, lambda, rhs, out, cs);
+  fdi_status st;
+  {
+    OwnCapture own(&p, 1);
+    st = field_solve(p, field, sigma, lambda, rhs, out, cs);
+  }
   cudaGraph_t gr = nullptr;
   cudaError_t e = cudaStreamEndCapture(cs, &gr);
   if (st != FDI_OK || e != cudaSuccess || gr == nullptr) {
@@ -513,7 +530,11 @@ fdi_status batch_solve(fdi_plan* const* plans, const double* lambdas, const doub
       const cudaStream_t cs = capture_stream(plans[0], s);
       if (!cs) return enqueue_batch(sp, plans, lambdas, rhs, out, count, s);
       FDI_CUDA_TRY(cudaStreamBeginCapture(cs, cudaStreamCaptureModeThreadLocal));
-      fdi_status st = enqueue_batch(sp, plans, lambdas, rhs, out, count, cs);
+      fdi_status st;
+      {
+        OwnCapture own(plans, count);
+        st = enqueue_batch(sp, plans, lambdas, rhs, out, count, cs);
+      }
       cudaGraph_t gr = nullptr;
       cudaError_t e = cudaStreamEndCapture(cs, &gr);
       cudaGraphExec_t ex = nullptr;

@@ -849,9 +849,7 @@ fdi_status stokes_solve(fdi_plan* p, double dt, double Re, const double* const f
       const long long body_start = p->launches;
       e = cudaStreamBeginCaptureToGraph(s, body, nullptr, nullptr, 0, cudaStreamCaptureModeThreadLocal);
       if (e == cudaSuccess) {
-        p->loop_capture = true;
         st = iteration(0);
-        p->loop_capture = false;
         if (st == FDI_OK) {
           k_loop_cond<<<1, 1, 0, s>>>(p->d_kry, h);
           p->launches++;
