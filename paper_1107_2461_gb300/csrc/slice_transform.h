@@ -38,7 +38,8 @@ fdi_status launch_slice_transform(fdi_plan* p, const SliceMatrix& m, const doubl
 // and ny are at most kSmallN, the three z steps of the TPF in one when nz is.
 // Whole solves, digit products against small kernels (us): TPT 16^3 53.6 / 35.0,
 // 24^3 59.6 / 39.1, 32^3 61.6 / 45.3, 40^3 69.9 / 67.6; TPF 16^3 61.6 / 30.9, 32^3
-// 67.8 / 41.1, 40^3 78.0 / 67.8; 24 x 24 x 256 148 / 131.  The plain multiply-adds
+// 67.8 / 41.1, 40^3 78.0 / 67.8; 24 x 24 x 256 148 / 131 (several digit planes per
+// MMA since took 40^3 to 67.8 TPT and 74.0 TPF).  The plain multiply-adds
 // grow as n^4, so the line is drawn at 32.
 constexpr int kSmallN = 32;
 bool small_plane_f64(const Field& f);
