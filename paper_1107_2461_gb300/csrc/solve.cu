@@ -58,10 +58,11 @@ fdi_status validate_field_args(const fdi_plan* p, int field, double sigma, doubl
 cudaGraph_t capturing_graph(cudaStream_t s) {
   cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
   cudaGraph_t g = nullptr;
-  if (cudaStreamGetCaptureInfo(s, &cap, nullptr, &g, nullptr, nullptr, nullptr) != cudaSuccess ||
-      cap != cudaStreamCaptureStatusActive)
+  if (cudaStreamGetCaptureInfo(s, &cap, nullptr, &g, nullptr, nullptr, nullptr) != cudaSuccess) {
+    cudaGetLastError();  // the legacy stream beside another stream's capture
     return nullptr;
-  return g;
+  }
+  return cap == cudaStreamCaptureStatusActive ? g : nullptr;
 }
 
 fdi_status graph_add_if(cudaStream_t s, cudaGraph_t g, cudaGraphConditionalHandle h, cudaGraph_t* body) {
@@ -163,8 +164,8 @@ fdi_status field_solve_internal(fdi_plan* p, int field, double sigma, double lam
   // the one before it, so a converged solve launches nothing more (a 16^3 solve
   // went from 80 to 58 us with its residual's reduction folded in, 64^3 from 127
   // to 105 us).
-  // Only in the graphs of field_solve_entry and batch_solve.  In a caller's own
-  // capture the rounds stay ordinary launches (a graph with conditional nodes
+  // Only in the graphs that field_solve_entry and batch_solve keep.  In a caller's
+  // own capture the rounds stay ordinary launches (a graph with conditional nodes
   // cannot be used everywhere a plain one can), and in the Krylov loop's WHILE
   // body too: there, with the solves joined from side streams right after their
   // conditional nodes, a replay never finished (the GPU idle, the host waiting).
@@ -290,13 +291,16 @@ bool same_key(const fdi_plan::GraphKey& a, const fdi_plan::GraphKey& b) {
 // eagerly, the second identical call is captured (stream capture of the same
 // launch sequence) and every later identical call is one graph launch.  The
 // cache keeps the graphs of the last few distinct argument sets.  Timed plans
-// need their events, so they run eagerly.
+// need their events, so they run eagerly.  A call on a stream that its caller is
+// capturing neither reads nor fills the cache: the launches themselves go into
+// the caller's graph (a kept graph would become a child of it, where conditional
+// nodes are not allowed, and no capture can begin inside another).
 fdi_status field_solve_entry(fdi_plan* p, int field, double sigma, double lambda, const double* rhs, double* out,
                              cudaStream_t s) {
   if (!p) return FDI_ERR_INVALID_ARG;
   p->launches = 0;
   p->kloop_body_launches = 0;
-  if (!p->use_graphs || p->timing) return field_solve(p, field, sigma, lambda, rhs, out, s);
+  if (!p->use_graphs || p->timing || capturing_graph(s)) return field_solve(p, field, sigma, lambda, rhs, out, s);
   fdi_plan::GraphKey key;
   key.field = field;
   key.sigma = sigma;
@@ -516,7 +520,7 @@ fdi_status batch_solve(fdi_plan* const* plans, const double* lambdas, const doub
     set_error("could not create the batch stream pool");
     return FDI_ERR_CUDA;
   }
-  bool graphs = true;
+  bool graphs = capturing_graph(s) == nullptr;  // a caller's capture gets the launches (field_solve_entry)
   for (int i = 0; i < count; ++i) graphs = graphs && plans[i]->use_graphs && !plans[i]->timing;
   std::lock_guard<std::mutex> lk(g_batch_mu);
   if (!graphs) return enqueue_batch(sp, plans, lambdas, rhs, out, count, s);
