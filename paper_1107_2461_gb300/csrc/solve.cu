@@ -280,6 +280,16 @@ struct OwnCapture {
   }
 };
 
+// While the library builds one of its graphs: another thread's capture (in the
+// global mode that PyTorch takes by default) forbids the stream creation and the
+// instantiation meant here and would be invalidated by them.  Nothing done in
+// this scope touches a stream of that capture.
+struct BesideCaptures {
+  cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+  BesideCaptures() { cudaThreadExchangeStreamCaptureMode(&mode); }
+  ~BesideCaptures() { cudaThreadExchangeStreamCaptureMode(&mode); }
+};
+
 bool same_key(const fdi_plan::GraphKey& a, const fdi_plan::GraphKey& b) {
   return a.field == b.field && a.sigma == b.sigma && a.lambda == b.lambda && a.rhs == b.rhs && a.out == b.out &&
          a.s == b.s;
@@ -340,6 +350,7 @@ fdi_status field_solve_entry(fdi_plan* p, int field, double sigma, double lambda
   }
   // second call with these arguments: capture, instantiate, launch
   g->last_use = ++p->gclock;
+  const BesideCaptures beside;
   const cudaStream_t cs = capture_stream(p, s);
   if (!cs) return field_solve(p, field, sigma, lambda, rhs, out, s);
   FDI_CUDA_TRY(cudaStreamBeginCapture(cs, cudaStreamCaptureModeThreadLocal));
@@ -531,6 +542,7 @@ fdi_status batch_solve(fdi_plan* const* plans, const double* lambdas, const doub
     g->last_use = ++g_batch_clock;
     if (!g->exec) {
       // second identical call: capture the fork / solves / join
+      const BesideCaptures beside;
       const cudaStream_t cs = capture_stream(plans[0], s);
       if (!cs) return enqueue_batch(sp, plans, lambdas, rhs, out, count, s);
       FDI_CUDA_TRY(cudaStreamBeginCapture(cs, cudaStreamCaptureModeThreadLocal));
