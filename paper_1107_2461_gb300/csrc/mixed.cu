@@ -211,24 +211,17 @@ __global__ void __launch_bounds__(256) k_init_rhs(ResidArgs a, SetupArgs w) {
       }
     }
   }
-  // within the warp in double-float (the FP64 pipe adds 2 lanes per clock)
-  df::F2 sb = df::make(sbb, 0.f);
+  // within the warp in FP64: the components packed over the lanes
+  const double ws = a.want_mean ? red::warp_sum4((double)sbb, df::to_f64(svb), df::to_f64(sv), 0.0)
+                                : red::warp_sum2((double)sbb, 0.0);
 #pragma unroll
-  for (int o = 16; o > 0; o >>= 1) {
-    sb = df::add(sb, df::make(__shfl_xor_sync(0xffffffffu, sb.hi, o), __shfl_xor_sync(0xffffffffu, sb.lo, o)));
-    rmax = fmaxf(rmax, __shfl_xor_sync(0xffffffffu, rmax, o));
-    if (a.want_mean) {
-      svb = df::add(svb, df::make(__shfl_xor_sync(0xffffffffu, svb.hi, o), __shfl_xor_sync(0xffffffffu, svb.lo, o)));
-      sv = df::add(sv, df::make(__shfl_xor_sync(0xffffffffu, sv.hi, o), __shfl_xor_sync(0xffffffffu, sv.lo, o)));
-    }
-  }
+  for (int o = 16; o > 0; o >>= 1) rmax = fmaxf(rmax, __shfl_xor_sync(0xffffffffu, rmax, o));
   if (lane == 0) {
-    sh[4 * warp] = 0.0;
-    sh[4 * warp + 1] = df::to_f64(sb);
-    sh[4 * warp + 2] = df::to_f64(svb);
-    sh[4 * warp + 3] = df::to_f64(sv);
+    sh[4 * warp + 1] = ws;
     smax[warp] = rmax;
   }
+  if (a.want_mean && lane == 16) sh[4 * warp + 2] = ws;
+  if (a.want_mean && lane == 8) sh[4 * warp + 3] = ws;
   __syncthreads();
   init_block_out(a, sh, smax, a.want_mean ? 4 : 2);
   finish_if_last(a.fin, threadIdx.x, blockDim.x);
