@@ -215,21 +215,6 @@ __device__ void thomas_singular_line(const ThomasArgs& a, const double* s_m, con
   }
 }
 
-// 1 / x from the hardware's coarse reciprocal (PTX rcp.approx.ftz.f64) and one step
-// of Householder's third-order iteration, x' = x + x (e + e^2), e = 1 - d x: the
-// error cubes (the seed's was at most 2^-19.9 over 5e8 values).  Three FP64
-// operations; the result was within 1 ulp of the correctly rounded one, and that
-// one itself for 99.4% of them.  The sweep is bound by the FP64 pipe: with lambda
-// Kd formed once per block and no FP64 -> FP32 conversion where nobody reads the
-// scale, 128^3 48 -> 44.5 us and a 24 x 24 x 256 solve 131 -> 122 us, a 256^3 solve
-// 1.69 -> 1.67 ms.
-__device__ __forceinline__ double rcp_f64(double d) {
-  double x;
-  asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(x) : "d"(d));
-  const double e = __fma_rn(-d, x, 1.0);
-  return __fma_rn(x, __fma_rn(e, e, e), x);
-}
-
 template <typename T, int kTP>
 __global__ void __launch_bounds__(128) k_thomas_f64(ThomasArgs a, const int* __restrict__ skip) {
   __shared__ double s_m[kMaxN], s_lo[kMaxN], s_kd[kMaxN];  // M_k, lambda K_{k,k+1}, lambda Kd_k
@@ -317,7 +302,7 @@ __global__ void __launch_bounds__(128) k_thomas_f64(ThomasArgs a, const int* __r
           const double up = (k + 1 < nz) ? -s_lo[k] : 0.0;
           double di = s * s_m[k] - s_kd[k];
           if (a.wy) di -= ly * a.wy[k];
-          const double inv = rcp_f64(di - lo * cprev);
+          const double inv = 1.0 / (di - lo * cprev);
           cprev = up * inv;
           // the same operations, in the same order, as the cached sweep: a
           // solve gives the same bits whether its factors were cached or not
