@@ -137,15 +137,17 @@ __device__ __forceinline__ void cp_async_wait() {
   asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory");
 }
 
-// x = +-m 2^(e - 1075) on a line whose largest biased exponent is eb, as the
+// x = +-m 2^(e - 1075) on a line whose largest biased exponent is eb >= 1, as the
 // fixed-point number round(x 2^(62 - (eb - 1022))), |.| < 2^62, plus 128 in every
-// base-256 digit: byte q of the result is digit 7 - q plus 128
+// base-256 digit: byte q of the result is digit 7 - q plus 128.  Zeros and
+// subnormal numbers have e = 1 and no leading bit.
 constexpr unsigned long long kDigitBias = 0x8080808080808080ull;
 __device__ __forceinline__ unsigned long long biased_digits(uint32_t lo, uint32_t hi, int eb) {
-  const int e = (int)((hi >> 20) & 0x7ffu);
-  unsigned long long m =
-      ((unsigned long long)(__funnelshift_l(lo, hi, 11) | 0x80000000u) << 32) | (unsigned long long)(lo << 11);
-  if (e == 0) m = 0;  // zero (and subnormals)
+  const uint32_t f = (hi >> 20) & 0x7ffu;
+  const int e = (int)max(f, 1u);
+  const unsigned long long m =
+      ((unsigned long long)((__funnelshift_l(lo, hi, 11) & 0x7fffffffu) | (min(f, 1u) << 31)) << 32) |
+      (unsigned long long)(lo << 11);
   const int sh = eb + 1 - e;  // >= 1; one extra bit, rounded away below
   unsigned long long y;
   asm("shr.u64 %0, %1, %2;" : "=l"(y) : "l"(m), "r"((unsigned)sh));  // 0 past 63 bits
@@ -583,7 +585,7 @@ __global__ void __launch_bounds__(THREADS, 1) k_slice_transform(const SliceArgs 
 #pragma unroll
           for (int l = 0; l < 8; ++l) {
             const uint32_t m = __reduce_max_sync(0xffffffffu, mx[l]);
-            if (lane == 0) s_exp[b * TN + LPW * w + l0 + l] = (int)(m >> 20);
+            if (lane == 0) s_exp[b * TN + LPW * w + l0 + l] = max((int)(m >> 20), 1);
           }
         }
       } else {
@@ -597,7 +599,7 @@ __global__ void __launch_bounds__(THREADS, 1) k_slice_transform(const SliceArgs 
         }
 #pragma unroll
         for (int o = LPW; o < 32; o <<= 1) mx = max(mx, __shfl_xor_sync(0xffffffffu, mx, o));
-        if (lane < LPW) s_exp[b * TN + LPW * w + line] = (int)(mx >> 20);
+        if (lane < LPW) s_exp[b * TN + LPW * w + line] = max((int)(mx >> 20), 1);
       }
       __syncwarp();
       if (lane == 0) tc::mbar_arrive(&expf_[b]);
@@ -624,7 +626,7 @@ __global__ void k_slice_matrix(const double* __restrict__ T, int n, int n_chunks
     if (k < n) mx = max(mx, (unsigned)__double2hiint(T[(size_t)k * n + j]) & 0x7fffffffu);
   atomicMax(&s_max, mx);
   __syncthreads();
-  const int eb = (int)(s_max >> 20);
+  const int eb = max((int)(s_max >> 20), 1);
   if (threadIdx.x == 0) row_exp[k] = eb;
   for (int j = threadIdx.x; j < n_chunks * TK; j += blockDim.x) {
     const double t = (k < n && j < n) ? T[(size_t)k * n + j] : 0.0;
