@@ -273,7 +273,7 @@ fdi_status fdi_apply_transform(fdi_plan* plan, fdi_field field, int d, int inver
 fdi_status fdi_eigen_noalloc(const double* faces, int n, int face_kind, fdi_bc bc_lo, fdi_bc bc_hi, double* lam,
                              double* E, double* Einv, int* converged, fdi_stream_t stream);
 
-/* Bound on every wait inside the kernels of a mixed plan that wait: the
+/* Bound on every wait inside the kernels of a plan that wait: the
  * tensor-core transforms (a CTA's roles hand shared-memory stages to one
  * another through mbarriers) and the grid barrier of the resident solve (its
  * CTAs meet between passes), in SM clock cycles; 0 restores the default of
@@ -285,8 +285,8 @@ fdi_status fdi_eigen_noalloc(const double* faces, int n, int face_kind, fdi_bc b
  * fdi_last_result (and every later solve's result) reports FDI_ERR_TIMEOUT,
  * until the next call of this function clears it.  The solution of a solve
  * that timed out is undefined.  Synchronises the device (the flag is cleared
- * once nothing runs); drops the plan's captured graphs.  FP64 plans accept
- * the call; the waits inside their transforms keep the default bound.
+ * once nothing runs); drops the plan's captured graphs.  Plans of either
+ * precision; FP64 plans wait in their transforms of more than 32 cells.
  * cycles < 0: FDI_ERR_INVALID_ARG. */
 fdi_status fdi_plan_set_wait_limit(fdi_plan* plan, long long cycles);
 

@@ -92,6 +92,7 @@ struct SliceArgs {
   long long slab, rs, ks;
   unsigned R, S;
   int n, m_tiles, n_chunks, n_items, accumulate;
+  long long wait_cycles;  // bound of every wait (cycles); 0: the default
 };
 
 // K-major operand with 32-byte rows in the 32-byte swizzle (8-row x 32-byte
@@ -250,7 +251,7 @@ __global__ void __launch_bounds__(THREADS, 1) k_slice_transform(const SliceArgs 
   int* s_exp = reinterpret_cast<int*>(smem + SM::EXP_OFF);  // [EXP_BUFS][TN]
   __shared__ volatile int s_abort;
   const int warp = __shfl_sync(0xffffffffu, threadIdx.x / 32, 0), lane = threadIdx.x % 32;
-  const long long wl = tc::kWaitCycles;
+  const long long wl = a.wait_cycles > 0 ? a.wait_cycles : tc::kWaitCycles;
 
   if (threadIdx.x == 0) {
     for (int s = 0; s < STAGES; ++s) {
@@ -291,6 +292,9 @@ __global__ void __launch_bounds__(THREADS, 1) k_slice_transform(const SliceArgs 
     const int b = g % GROUPS, phase = g / GROUPS - (b < STAGES ? 1 : 0);
     return tc::mbar_wait(&freed[b], (uint32_t)(phase & 1), &s_abort, wl);
   };
+  // a wait of a whole warp: after a time-out its lanes leave together (a lane may
+  // see the phase complete while another sees the abort flag)
+  auto together = [](bool ok) -> bool { return __all_sync(0xffffffffu, ok) != 0; };
 
   if (warp == 0) {
     if (tc::elect_one()) {
@@ -419,8 +423,8 @@ __global__ void __launch_bounds__(THREADS, 1) k_slice_transform(const SliceArgs 
     double* tp = reinterpret_cast<double*>(smem + SM::EPI_OFF + ww * EPI_BYTES);
     auto epilogue = [&](int it) -> bool {
       const int lt = (i0 + it) / a.m_tiles, mt = (i0 + it) % a.m_tiles, ltq = lt - lt0, eb_buf = ltq % EXP_BUFS;
-      if (!tc::mbar_wait(&expf_[eb_buf], (ltq / EXP_BUFS) & 1, &s_abort, wl) ||
-          !tc::mbar_wait(accf, (uint32_t)(it & 1), &s_abort, wl)) {
+      if (!together(tc::mbar_wait(&expf_[eb_buf], (ltq / EXP_BUFS) & 1, &s_abort, wl) &&
+                    tc::mbar_wait(accf, (uint32_t)(it & 1), &s_abort, wl))) {
         atomicExch(a.err, 5);
         return false;
       }
@@ -506,7 +510,7 @@ __global__ void __launch_bounds__(THREADS, 1) k_slice_transform(const SliceArgs 
     issue(grp);
     int it = grp / nK, kc = grp % nK, ltq = -1, eb = 0, done = 0;
     bool ok = true;
-    for (int gi = grp; gi < total && !s_abort; gi += GROUPS) {
+    for (int gi = grp; gi < total; gi += GROUPS) {
       while (done < items && gi >= (done + 1) * nK + STAGES && ok) ok = epilogue(done++);
       if (!ok) break;
       const int s = gi % STAGES;
@@ -521,13 +525,13 @@ __global__ void __launch_bounds__(THREADS, 1) k_slice_transform(const SliceArgs 
       const int want = (i0 + it) / a.m_tiles - lt0;
       if (want != ltq) {
         ltq = want;
-        ok = tc::mbar_wait(&expf_[ltq % EXP_BUFS], (ltq / EXP_BUFS) & 1, &s_abort, wl);
+        ok = together(tc::mbar_wait(&expf_[ltq % EXP_BUFS], (ltq / EXP_BUFS) & 1, &s_abort, wl));
         eb = s_exp[(ltq % EXP_BUFS) * TN + 16 * wg + line];
       }
       unsigned long long u[8];
 #pragma unroll
       for (int q = 0; q < 8; ++q) u[q] = biased_digits(x[q].x, x[q].y, eb);
-      if (!ok || !stage_free(gi)) {
+      if (!ok || !together(stage_free(gi))) {
         atomicExch(a.err, 4);
         break;
       }
@@ -554,7 +558,7 @@ __global__ void __launch_bounds__(THREADS, 1) k_slice_transform(const SliceArgs 
         ++it;
       }
     }
-    while (done < items && ok && !s_abort) ok = epilogue(done++);
+    while (done < items && ok) ok = epilogue(done++);
     cp_async_wait<0>();
   } else {
     // ---------------- line exponents ----------------
@@ -564,9 +568,9 @@ __global__ void __launch_bounds__(THREADS, 1) k_slice_transform(const SliceArgs 
     const int w = warp - W_EXP;
     const int last = items > 0 ? (i0 + items - 1) / a.m_tiles - lt0 : -1;
     const uint32_t* hi = reinterpret_cast<const uint32_t*>(a.in) + 1;
-    for (int ltq = 0; ltq <= last && !s_abort; ++ltq) {
+    for (int ltq = 0; ltq <= last; ++ltq) {
       const int b = ltq % EXP_BUFS;
-      if (!tc::mbar_wait(&expe[b], ((ltq / EXP_BUFS) & 1) ^ 1, &s_abort, wl)) {
+      if (!together(tc::mbar_wait(&expe[b], ((ltq / EXP_BUFS) & 1) ^ 1, &s_abort, wl))) {
         atomicExch(a.err, 6);
         break;
       }
@@ -699,6 +703,7 @@ fdi_status launch_slice_transform(fdi_plan* p, const SliceMatrix& m, const doubl
   a.m_tiles = m.m_tiles;
   a.n_chunks = m.n_chunks;
   a.accumulate = accumulate ? 1 : 0;
+  a.wait_cycles = p->wait_cycles;
   int sms = 152;
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, p->device);
   // 64 lines per item, or 32 where that leaves SMs without work
