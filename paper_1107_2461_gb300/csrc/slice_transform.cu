@@ -2,7 +2,7 @@
 //
 // One pass of the FP64 path (Sec. 3, Eq. 25/29) applies a dense n x n matrix T
 // (E_d^{-1} or E_d) to every grid line of direction d.  GB300 multiplies FP64 at
-// 2 FMA/clk/SM, so on the FP64 pipe a 256^3 pass takes 6.9 ms (34 GFLOP at 1.25
+// 2 FMA/clk/SM, so on the FP64 pipe a 256^3 pass takes 6.9 ms (8.6 GFLOP at 1.25
 // TFLOP/s); the same product of digits runs at the fp16 tensor rate.
 //
 // Method (Ozaki, Ogita, Oishi, Rump, Numer. Algorithms 59, 2012: error-free
@@ -12,15 +12,25 @@
 // [-128, 128), the leading one in [-64, 64]); the rows of T are split the same
 // way at plan time.  Digits are exact in fp16, their products and the FP32 sums
 // of products are integers:
-//     S_L = sum_{u + v = L} sum_j T^(u)[k][j] x^(v)[j],   L = 0 .. 7.
-// For n <= 256 the bounds of |S_0| .. |S_4| are 2^20, 2^22, 2^23, 2^23.6 and
-// 2^24, so these are exact for any input; a rounding of S_5 .. S_7 (only when
-// they pass 2^24) is below 2^-58 of max |T| max |x|.  The 36 products u + v <= 7
-// leave out terms of 2^-60.  The sums are added as integers and rounded to FP64
-// once: on the lines of a 256-cell direction the error is 0.1-1.2 times that of
-// a chain of 256 FP64 multiply-adds (5e-17 relative for lines with a decaying
-// spectrum, where both are one rounding of the result; 5e-17 against 4.7e-16
-// for uniform ones).  Seven digits were not enough: 2e-15 on decaying lines.
+//     S_L = sum_{u + v = L} sum_j T^(u)[k][j] x^(v)[j],   L = 0 .. 7,
+// in units of 2^(-12 - 8 L) of the scale (the product of the powers of two above
+// the line's and the row's largest entries).  For n <= 256 the bounds of
+// |S_0| .. |S_4| are 2^20, 2^22, 2^23, 2^23.6 and 2^24, so these are exact for any
+// input.  S_5 .. S_7 can pass 2^24 (up to 2^24.8), but only when the digits are
+// near 128 and of one sign in nearly all of 256 columns (sums of random digits are
+// 2^18 in root mean square); an FP32 sum then rounds by a unit, for S_5 2^-52 of the
+// scale, of which the result itself is at least 2^-6.  The 36 products u + v <= 7
+// leave out S_8 and beyond, 2^-58 of the scale in root mean square over 256 columns.
+// The sums are added as integers and rounded to FP64 once.
+//
+// Accuracy is relative to the largest entry of a line, which is what the norm of a
+// solution sees: on a 128-cell direction the error in a line's norm is 4-6e-17,
+// that of a chain of FP64 multiply-adds 2-3e-16.  An entry 2^-k below the largest
+// keeps 62 - k bits, so single results far below it are less exact than a chain's:
+// the spectral coefficients of a narrow bump, half of them below 2e-16 of the
+// largest, have a median relative error of 1e-3 against 1e-12.  Through the whole
+// inverse the two agree point by point, since the errors of the eigenvectors weigh
+// more.  Seven digits were not enough: 2e-15 on decaying lines.
 //
 // Layout: T is the MMA's A operand (M = 128 output modes), 64 grid lines are
 // its B operand (N = 64): eight FP32 accumulators of 64 columns fill tensor
