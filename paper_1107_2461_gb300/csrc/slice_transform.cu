@@ -122,16 +122,6 @@ __host__ __device__ __forceinline__ uint32_t sw32_offset(int row, int h) {
   return (uint32_t)(row * 32 + ((h ^ ((row >> 2) & 1)) << 4));
 }
 
-// digit planes of the lines times one digit plane of T
-__device__ __forceinline__ void mma_digits(uint32_t d, uint64_t a, uint64_t b, uint32_t idesc, uint32_t acc) {
-  asm volatile(
-      "{\n\t.reg .pred p;\n\t"
-      "setp.ne.b32 p, %4, 0;\n\t"
-      "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}" ::"r"(d),
-      "l"(a), "l"(b), "r"(idesc), "r"(acc)
-      : "memory");
-}
-
 __device__ __forceinline__ void tmem_ld4(uint32_t taddr, float (&r)[4]) {
   asm volatile("tcgen05.ld.sync.aligned.32x32b.x4.b32 {%0, %1, %2, %3}, [%4];"
                : "=f"(r[0]), "=f"(r[1]), "=f"(r[2]), "=f"(r[3])
@@ -361,7 +351,7 @@ __global__ void __launch_bounds__(THREADS, 1) k_slice_transform(const SliceArgs 
               const int planes = SL - u - v < NPL ? SL - u - v : NPL;
               const uint32_t d = tmem + (uint32_t)((u + v) * TN);
               const uint64_t db = sdesc_k_sw32(sb + v * SM::B_SLICE);
-              mma_digits(d, da, db, tc::idesc_f16_f32(TM, planes * TN), acc);
+              tc::mma_f16(d, da, db, tc::idesc_f16_f32(TM, planes * TN), acc);
             }
           }
           tc::mma_commit(&freed[(g + STAGES) % GROUPS]);

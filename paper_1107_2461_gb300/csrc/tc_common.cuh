@@ -99,20 +99,9 @@ __device__ __forceinline__ void tma_store_2d(const CUtensorMap* map, uint32_t sr
                "r"(c0), "r"(c1), "r"(src)
                : "memory");
 }
-__device__ __forceinline__ void tma_store_3d(const CUtensorMap* map, uint32_t src, int c0, int c1, int c2) {
-  asm volatile("cp.async.bulk.tensor.3d.global.shared::cta.bulk_group [%0, {%1, %2, %3}], [%4];" ::"l"(
-                   reinterpret_cast<uint64_t>(map)),
-               "r"(c0), "r"(c1), "r"(c2), "r"(src)
-               : "memory");
-}
 __device__ __forceinline__ void bulk_commit() { asm volatile("cp.async.bulk.commit_group;" ::: "memory"); }
 // every committed bulk store of this thread has finished reading shared memory
 __device__ __forceinline__ void bulk_wait_read_all() { asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory"); }
-// all but the most recently committed bulk store of this thread have finished
-// reading shared memory
-__device__ __forceinline__ void bulk_wait_read_1() { asm volatile("cp.async.bulk.wait_group.read 1;" ::: "memory"); }
-// every committed bulk store of this thread has completed
-__device__ __forceinline__ void bulk_wait_all() { asm volatile("cp.async.bulk.wait_group 0;" ::: "memory"); }
 
 __device__ __forceinline__ void prefetch_tmap(const CUtensorMap* map) {
   asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(map)) : "memory");
@@ -186,18 +175,7 @@ __device__ __forceinline__ void tmem_ld32(uint32_t taddr, uint32_t (&r)[32]) {
 __device__ __forceinline__ void tmem_ld_wait() { asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory"); }
 
 // Shared-memory matrix descriptor (tcgen05 format): K-major operand stored in
-// the 128-byte swizzle layout (8-row x 128-byte atoms, 1024 bytes apart).
-__device__ __forceinline__ uint64_t sdesc_k_sw128(uint32_t saddr) {
-  uint64_t d = 0;
-  d |= (uint64_t)((saddr & 0x3FFFF) >> 4);          // start address, bits 0-13
-  d |= (uint64_t)1 << 16;                           // leading byte offset (unused for swizzled K-major)
-  d |= (uint64_t)(1024 >> 4) << 32;                 // stride byte offset: next 8-row group
-  d |= (uint64_t)1 << 46;                           // descriptor version (sm_100 family)
-  d |= (uint64_t)2 << 61;                           // layout: 128-byte swizzle
-  return d;
-}
-
-// Same for the 64-byte swizzle layout (8-row x 64-byte atoms, 512 bytes apart).
+// the 64-byte swizzle layout (8-row x 64-byte atoms, 512 bytes apart).
 __device__ __forceinline__ uint64_t sdesc_k_sw64(uint32_t saddr) {
   uint64_t d = 0;
   d |= (uint64_t)((saddr & 0x3FFFF) >> 4);          // start address, bits 0-13
@@ -215,13 +193,6 @@ __host__ __device__ constexpr uint32_t idesc_f16_f32(int M, int N) {
          | (0u << 10)                    // B format: f16
          | ((uint32_t)(N >> 3) << 17)    // N / 8
          | ((uint32_t)(M >> 4) << 24);   // M / 16
-}
-
-// byte offset of element (row, k) of a K-major fp16 tile with 64 fp16 per
-// 128-byte row in the 128-byte swizzle layout
-__device__ __forceinline__ uint32_t sw128_offset(int row, int k) {
-  int chunk = k >> 3;  // 16-byte chunk (8 fp16)
-  return (uint32_t)(row * 128 + ((chunk ^ (row & 7)) << 4) + ((k & 7) << 1));
 }
 
 // byte offset of element (row, k) of a K-major fp16 tile with 32 fp16 per

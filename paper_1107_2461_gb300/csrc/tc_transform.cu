@@ -58,7 +58,6 @@ constexpr int NGRP = NCONV / 2;
 constexpr int NEPI = 8;                       // two per tensor-memory quarter, alternate 32-column blocks
 constexpr int WARP_A = 2 + NCONV + NEPI;      // A producer warp
 constexpr int THREADS = 32 * (WARP_A + 1);
-constexpr bool kTmaTransposed = false;
 constexpr int EPI_WARP_BYTES = 4 * 1024;      // per epilogue warp: one 32 x 32 block (transpose tile or TMA staging)
 constexpr int TP_BYTES = NEPI * EPI_WARP_BYTES;
 constexpr int BAR_BYTES = 256;
@@ -470,35 +469,22 @@ __global__ void __launch_bounds__(THREADS, 1)
           // read the tile (the other seven warps work meanwhile).
           if (lane == 0) tc::bulk_wait_read_all();
           __syncwarp();
-          if (a.tma_store == 1) {
-            // staging [column][row]: 32 rows of one column are 128 contiguous bytes
+          // staging [row][column] in the 128-byte swizzle (16-byte unit u of row
+          // `lane` at unit u ^ (lane & 7))
 #pragma unroll
-            for (int j = 0; j < 32; ++j) {
-              const float v = __uint_as_float(r[j]) * s_cs[c0 + j];
-              vmax = fmaxf(vmax, fabsf(v));
-              tp[j * 32 + lane] = v;
-            }
-          } else {
-            // staging [row][column] in the 128-byte swizzle (16-byte unit u of row
-            // `lane` at unit u ^ (lane & 7))
-#pragma unroll
-            for (int u = 0; u < 8; ++u) {
-              const float4 cs = *reinterpret_cast<const float4*>(s_cs + c0 + 4 * u);
-              const float4 v = make_float4(__uint_as_float(r[4 * u]) * cs.x, __uint_as_float(r[4 * u + 1]) * cs.y,
-                                           __uint_as_float(r[4 * u + 2]) * cs.z, __uint_as_float(r[4 * u + 3]) * cs.w);
-              vmax = fmaxf(fmaxf(vmax, fmaxf(fabsf(v.x), fabsf(v.y))), fmaxf(fabsf(v.z), fabsf(v.w)));
-              *reinterpret_cast<float4*>(tp + lane * 32 + ((u ^ (lane & 7)) << 2)) = v;
-            }
+          for (int u = 0; u < 8; ++u) {
+            const float4 cs = *reinterpret_cast<const float4*>(s_cs + c0 + 4 * u);
+            const float4 v = make_float4(__uint_as_float(r[4 * u]) * cs.x, __uint_as_float(r[4 * u + 1]) * cs.y,
+                                         __uint_as_float(r[4 * u + 2]) * cs.z, __uint_as_float(r[4 * u + 3]) * cs.w);
+            vmax = fmaxf(fmaxf(vmax, fmaxf(fabsf(v.x), fabsf(v.y))), fmaxf(fabsf(v.z), fabsf(v.w)));
+            *reinterpret_cast<float4*>(tp + lane * 32 + ((u ^ (lane & 7)) << 2)) = v;
           }
           tc::fence_proxy_async_smem();
           __syncwarp();
           if (nrows > 0) {
             if (lane == 0) {
               const uint32_t stg = tc::smem_u32(tp);  // 1024-byte aligned
-              if (a.tma_store == 1)
-                tc::tma_store_3d(&tmO, stg, (int)(wrow0 % a.S), c0, (int)(wrow0 / a.S));
-              else
-                tc::tma_store_2d(&tmO, stg, c0, (int)wrow0);
+              tc::tma_store_2d(&tmO, stg, c0, (int)wrow0);
               tc::bulk_commit();
             }
           }
@@ -787,35 +773,24 @@ fdi_status launch_tc_transform(fdi_plan* p, const TcMatrix& m, TcArgs args, cons
       return FDI_ERR_CUDA;
     }
   }
-  // output through TMA stores where the layout allows: 16-byte aligned base and
-  // strides, and (transposed outputs) slabs made of whole 32-row warp blocks
+  // row-major output through TMA stores where the layout allows (16-byte aligned
+  // base and strides); transposed outputs keep the thread stores (16-byte row groups
+  // after an in-shared transpose), which measured faster than 32 x 32 TMA boxes of
+  // 128-byte column segments
   CUtensorMap mapO;
   memset(&mapO, 0, sizeof(mapO));
   args.tma_store = 0;
   const bool out_aligned = (reinterpret_cast<uintptr_t>(args.out_f32) & 15u) == 0;
-  if (args.mode == TC_OUT_F32 && out_aligned && args.n_out > 0) {
-    cuuint32_t estr[3] = {1, 1, 1};
-    // transposed outputs keep the thread stores (16-byte row groups after an
-    // in-shared transpose), which measured faster than 32 x 32 TMA boxes of
-    // 128-byte column segments; kTmaTransposed enables the TMA variant
-    if (kTmaTransposed && args.row_stride == 1 && args.S % 32 == 0 && args.R % args.S == 0 &&
-        args.col_stride % 4 == 0 && args.slab_stride % 4 == 0 && args.R / args.S < 0x7fffffffLL) {
-      cuuint64_t dims[3] = {(cuuint64_t)args.S, (cuuint64_t)args.n_out, (cuuint64_t)(args.R / args.S)};
-      cuuint64_t strides[2] = {(cuuint64_t)args.col_stride * sizeof(float), (cuuint64_t)args.slab_stride * sizeof(float)};
-      cuuint32_t box[3] = {32, 32, 1};
-      if (enc(&mapO, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 3, args.out_f32, dims, strides, box, estr,
-              CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_NONE,
-              CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS)
-        args.tma_store = 1;
-    } else if (args.col_stride == 1 && args.S == args.R && args.row_stride % 4 == 0 && args.row_stride >= args.n_out) {
-      cuuint64_t dims[2] = {(cuuint64_t)args.n_out, (cuuint64_t)args.R};
-      cuuint64_t strides[1] = {(cuuint64_t)args.row_stride * sizeof(float)};
-      cuuint32_t box[2] = {32, 32};
-      if (enc(&mapO, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 2, args.out_f32, dims, strides, box, estr,
-              CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_NONE,
-              CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS)
-        args.tma_store = 2;
-    }
+  if (args.mode == TC_OUT_F32 && out_aligned && args.n_out > 0 && args.col_stride == 1 && args.S == args.R &&
+      args.row_stride % 4 == 0 && args.row_stride >= args.n_out) {
+    cuuint32_t estr[2] = {1, 1};
+    cuuint64_t dims[2] = {(cuuint64_t)args.n_out, (cuuint64_t)args.R};
+    cuuint64_t strides[1] = {(cuuint64_t)args.row_stride * sizeof(float)};
+    cuuint32_t box[2] = {32, 32};
+    if (enc(&mapO, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 2, args.out_f32, dims, strides, box, estr,
+            CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_NONE,
+            CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS)
+      args.tma_store = 1;
   }
   return launch_kernel(p, m, mapA, mapO, args, tiles, s);
 }
