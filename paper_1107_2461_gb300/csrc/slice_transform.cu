@@ -292,9 +292,6 @@ __global__ void __launch_bounds__(THREADS, 1) k_slice_transform(const SliceArgs 
     const int b = g % GROUPS, phase = g / GROUPS - (b < STAGES ? 1 : 0);
     return tc::mbar_wait(&freed[b], (uint32_t)(phase & 1), &s_abort, wl);
   };
-  // a wait of a whole warp: after a time-out its lanes leave together (a lane may
-  // see the phase complete while another sees the abort flag)
-  auto together = [](bool ok) -> bool { return __all_sync(0xffffffffu, ok) != 0; };
 
   if (warp == 0) {
     if (tc::elect_one()) {
@@ -423,8 +420,8 @@ __global__ void __launch_bounds__(THREADS, 1) k_slice_transform(const SliceArgs 
     double* tp = reinterpret_cast<double*>(smem + SM::EPI_OFF + ww * EPI_BYTES);
     auto epilogue = [&](int it) -> bool {
       const int lt = (i0 + it) / a.m_tiles, mt = (i0 + it) % a.m_tiles, ltq = lt - lt0, eb_buf = ltq % EXP_BUFS;
-      if (!together(tc::mbar_wait(&expf_[eb_buf], (ltq / EXP_BUFS) & 1, &s_abort, wl) &&
-                    tc::mbar_wait(accf, (uint32_t)(it & 1), &s_abort, wl))) {
+      if (!tc::together(tc::mbar_wait(&expf_[eb_buf], (ltq / EXP_BUFS) & 1, &s_abort, wl) &&
+                        tc::mbar_wait(accf, (uint32_t)(it & 1), &s_abort, wl))) {
         atomicExch(a.err, 5);
         return false;
       }
@@ -525,13 +522,13 @@ __global__ void __launch_bounds__(THREADS, 1) k_slice_transform(const SliceArgs 
       const int want = (i0 + it) / a.m_tiles - lt0;
       if (want != ltq) {
         ltq = want;
-        ok = together(tc::mbar_wait(&expf_[ltq % EXP_BUFS], (ltq / EXP_BUFS) & 1, &s_abort, wl));
+        ok = tc::together(tc::mbar_wait(&expf_[ltq % EXP_BUFS], (ltq / EXP_BUFS) & 1, &s_abort, wl));
         eb = s_exp[(ltq % EXP_BUFS) * TN + 16 * wg + line];
       }
       unsigned long long u[8];
 #pragma unroll
       for (int q = 0; q < 8; ++q) u[q] = biased_digits(x[q].x, x[q].y, eb);
-      if (!ok || !together(stage_free(gi))) {
+      if (!ok || !tc::together(stage_free(gi))) {
         atomicExch(a.err, 4);
         break;
       }
@@ -570,7 +567,7 @@ __global__ void __launch_bounds__(THREADS, 1) k_slice_transform(const SliceArgs 
     const uint32_t* hi = reinterpret_cast<const uint32_t*>(a.in) + 1;
     for (int ltq = 0; ltq <= last; ++ltq) {
       const int b = ltq % EXP_BUFS;
-      if (!together(tc::mbar_wait(&expe[b], ((ltq / EXP_BUFS) & 1) ^ 1, &s_abort, wl))) {
+      if (!tc::together(tc::mbar_wait(&expe[b], ((ltq / EXP_BUFS) & 1) ^ 1, &s_abort, wl))) {
         atomicExch(a.err, 6);
         break;
       }

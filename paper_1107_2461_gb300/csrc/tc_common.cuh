@@ -63,6 +63,12 @@ __device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity, volati
   return true;
 }
 
+// Outcome of a wait that every lane of a warp made: the same in all lanes, so that
+// after a time-out they leave together (one lane may see the phase complete while
+// another sees the abort flag, and the rest of the warp would wait for it at the
+// next warp barrier).
+__device__ __forceinline__ bool together(bool ok) { return __all_sync(0xffffffffu, ok) != 0; }
+
 // Wait for a phase that is certain to complete (an issued TMA load, a
 // committed MMA batch), ignoring `abort`: used after a failure to drain the
 // asynchronous operations of this CTA before it frees TMEM and exits.  Still

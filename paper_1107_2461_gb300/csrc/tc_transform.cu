@@ -325,9 +325,9 @@ __global__ void __launch_bounds__(THREADS, 1)
     const bool a_mn = a.a_mn != 0;
     const int c8 = ct & 3, r4 = ct >> 2;
     int kc = grp % nK;
-    for (uint32_t g = grp; g < total && !s_abort; g += 2) {
+    for (uint32_t g = grp; g < total; g += 2) {
       const int sa = g % NA32, s = g % NS;
-      if (!tc::mbar_wait(&a_full[sa], (g / NA32) & 1, &s_abort, wl)) {
+      if (!tc::together(tc::mbar_wait(&a_full[sa], (g / NA32) & 1, &s_abort, wl))) {
         atomicExch(a.err, 4);
         break;
       }
@@ -350,7 +350,7 @@ __global__ void __launch_bounds__(THREADS, 1)
 #pragma unroll
           for (int e = 0; e < 8; ++e) v[q][e] = sf[(8 * q + e) * BM + ct];
       }
-      if (!tc::mbar_wait(&empty_a[s], ((g / NS) & 1) ^ 1, &s_abort, wl)) {
+      if (!tc::together(tc::mbar_wait(&empty_a[s], ((g / NS) & 1) ^ 1, &s_abort, wl))) {
         atomicExch(a.err, 4);
         break;
       }
@@ -431,13 +431,13 @@ __global__ void __launch_bounds__(THREADS, 1)
                        (reinterpret_cast<uintptr_t>(a.out_f32) & 15u) == 0;
     const int g8 = lane >> 3, l8 = lane & 7;  // after the transpose: group of 8 lanes, lane in group
     float vmax = 0.f;
-    for (int it = 0; it < my_iters && !s_abort; ++it) {
+    for (int it = 0; it < my_iters; ++it) {
       int half = -1;
       const int tile = item_tile(it, &half);
       const int c_lo = half == 1 ? N_pad / 2 : 0, c_hi = half == 0 ? N_pad / 2 : N_pad;
       const int buf = (int)(it & 1);
       const uint32_t aph = (uint32_t)((it >> 1) & 1);
-      if (!tc::mbar_wait(&accf[buf], aph, &s_abort, wl)) {
+      if (!tc::together(tc::mbar_wait(&accf[buf], aph, &s_abort, wl))) {
         atomicExch(a.err, 5);
         break;
       }
