@@ -76,7 +76,8 @@ typedef enum { FDI_GRID_CELL = 0, FDI_GRID_MAC = 1 } fdi_grid;
 
 /* Arithmetic of the x/y eigenvector transforms (the dense contractions of
  * Eq. 25/29).  FDI_PREC_FP64: every step in FP64 (the transforms as exact
- * products of 62-bit fixed-point digits, rounded to FP64 once).  The mixed modes split each
+ * products of 62-bit fixed-point digits, scaled to the largest entry of each
+ * grid line, rounded to FP64 once).  The mixed modes split each
  * operand into a high and a low part in a 16-bit (or TF32) tensor-core type,
  * form hi*hi + hi*lo + lo*hi with FP32 accumulation, keep the intermediate
  * fields in FP32, run the Thomas sweep in FP32, and recover FP64 accuracy by
@@ -339,7 +340,9 @@ fdi_status fdi_plan_autotune(fdi_plan* plan, double lambda, const double* rhs, d
  * second occurrence and replayed as one graph launch from then on; results are
  * identical to the eager launch sequence.  A default stream cannot be captured:
  * solves called on it are captured on a stream of the plan's and the graph is
- * launched on the caller's.  Plans with timing on always run eagerly.  Changing tolerances or the Thomas
+ * launched on the caller's.  Into a stream that the caller is capturing the
+ * launches themselves are enqueued, whatever graphs are kept.  Plans with
+ * timing on always run eagerly.  Changing tolerances or the Thomas
  * configuration drops the captured graph.  on: 0 off, nonzero on. */
 fdi_status fdi_plan_set_graphs(fdi_plan* plan, int on);
 

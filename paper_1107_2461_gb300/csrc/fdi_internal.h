@@ -112,7 +112,7 @@ struct fdi_plan {
   int thomas_tl = 2;                // FP32 Thomas: lines per CTA (64, 128) or 2 = two lines per thread
   float2* lam_w = nullptr;          // lambda-scaled double-float flux weights [3][3][kMaxN]
   unsigned* d_counter = nullptr;    // ticket counter of the fused last-block reductions (zero between launches)
-  cudaStream_t cstream = nullptr;   // mixed plans: captures the bodies of conditional refinement rounds
+  cudaStream_t cstream = nullptr;   // captures the bodies of conditional refinement rounds
   double* partials = nullptr;       // reduction partials
   int npartials = 0;
   // Thomas factor cache of this workspace: the reciprocal pivots and c' of
@@ -328,7 +328,7 @@ fdi_status eigen_decompose_batch(int count, int n, const double* m, const double
 
 // FP64 path launchers (kernels_f64.cu).  Transform of direction d of a field by
 // E_d^{-1} (forward) or E_d: out (+)= T in along every line of d (x lines may
-// accumulate), on the tensor cores or the FP64 pipe
+// accumulate), on the tensor cores (digit products)
 // (pdl: programmatic launch; not for the first kernel after a graph's
 // conditional node, a join or a copy)
 fdi_status launch_axis_f64(fdi_plan* p, const Field& f, int d, bool forward, const double* in, double* out,

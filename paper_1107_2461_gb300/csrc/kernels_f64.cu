@@ -8,8 +8,9 @@
 //                 end of Sec. 3: Thomas algorithm in one direction)
 //   k_divide_f64  u_ijk = f_ijk / (sigma - lam (Lx_i + Ly_j + Lz_k))  (Eq. 26-28)
 //   k_residual_f64 r = b - A u with the 7-point finite-volume stencil in flux form,
-//                 and per-block partial sums of r^2 and b^2 (fixed grid, so the
-//                 reduction order is deterministic)
+//                 the sums of r^2 and b^2 (per-block partial sums, added by the
+//                 block that finishes last in a fixed order) and the convergence
+//                 check
 //
 // GB300 runs FP64 at about 2 FMA/clk/SM, so k_slab_f64 is FP64-pipe bound; it is
 // register-tiled (4x4 outputs per thread, 64x64 tiles staged in shared
