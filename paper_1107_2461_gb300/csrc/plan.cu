@@ -120,6 +120,7 @@ fdi_status dev_alloc(T** p, size_t count) {
   if (count == 0) count = 1;
   cudaError_t e = cudaMalloc((void**)p, count * sizeof(T));
   if (e != cudaSuccess) {
+    cudaGetLastError();  // reported here, not by the next launch check
     set_error(std::string("cudaMalloc: ") + cudaGetErrorString(e));
     *p = nullptr;
     return e == cudaErrorMemoryAllocation ? FDI_ERR_OUT_OF_MEMORY : FDI_ERR_CUDA;

@@ -651,8 +651,13 @@ fdi_status prepare_matrix(fdi_plan* p, const double* T, int n, SliceMatrix* m, c
   m->n = n;
   m->m_tiles = (n + TM - 1) / TM;
   m->n_chunks = (n + TK - 1) / TK;
-  FDI_CUDA_TRY(cudaMalloc(&m->img, (size_t)m->m_tiles * m->n_chunks * A_BYTES));
-  FDI_CUDA_TRY(cudaMalloc(&m->row_exp, (size_t)m->m_tiles * TM * sizeof(int)));
+  cudaError_t e = cudaMalloc(&m->img, (size_t)m->m_tiles * m->n_chunks * A_BYTES);
+  if (e == cudaSuccess) e = cudaMalloc(&m->row_exp, (size_t)m->m_tiles * TM * sizeof(int));
+  if (e != cudaSuccess) {
+    cudaGetLastError();  // reported here, not by the next launch check
+    set_error(std::string("digit planes of a transform: ") + cudaGetErrorString(e));
+    return e == cudaErrorMemoryAllocation ? FDI_ERR_OUT_OF_MEMORY : FDI_ERR_CUDA;
+  }
   k_slice_matrix<<<m->m_tiles * TM, 256, 0, s>>>(T, n, m->n_chunks, m->img, m->row_exp);
   FDI_LAUNCH_CHECK(p);
   return FDI_OK;

@@ -5,6 +5,17 @@
 #include "fdi_internal.h"
 #include "slice_transform.h"
 
+// status of preparing an n x n matrix, n so large that its digit planes exceed any
+// device memory: the allocation is refused before anything reads T
+extern "C" int slice_prepare_status(int n) {
+  fdi_plan p;
+  fdi::Axis ax;
+  ax.n = n;
+  const int st = (int)fdi::slice_prepare_axis(&p, &ax, nullptr);
+  fdi::slice_free_axis(&ax);
+  return st;
+}
+
 extern "C" int slice_transform_check(const double* T, int n, const double* in, double* out, long long lines,
                                      int contiguous, long long width, int accumulate) {
   fdi_plan p;

@@ -42,9 +42,11 @@ def check(tmp_path_factory):
     subprocess.run([build.nvcc()] + build.ARCH + build.NVCC_FLAGS +
                    ["-I" + build.CSRC, "-shared", os.path.join(HERE, "slice_transform_check.cu"), lib, "-o", out,
                     "-Xlinker", "-rpath," + os.path.dirname(lib)], check=True)
-    fn = C.CDLL(out).slice_transform_check
+    so = C.CDLL(out)
+    fn = so.slice_transform_check
     fn.restype = C.c_int
     fn.argtypes = [C.c_void_p, C.c_int, C.c_void_p, C.c_void_p, C.c_longlong, C.c_int, C.c_longlong, C.c_int]
+    fn.prepare_status = so.slice_prepare_status
     return fn
 
 
@@ -173,3 +175,17 @@ def test_against_exact_sums(check, n, lines, kind, contiguous):
     # adding to what is there: 3 y after two more passes
     apply(1)
     assert np.array_equal(apply(1), (y + y) + y)
+
+
+def test_out_of_memory_is_reported_once(check):
+    import torch
+    from paper_1107_2461_gb300 import ERR_OUT_OF_MEMORY
+    assert check.prepare_status(1 << 20) == ERR_OUT_OF_MEMORY  # 17 TB
+    # the next launch does not report it again
+    eye = torch.eye(33, dtype=torch.float64, device="cuda")
+    x = torch.randn(5, 33, dtype=torch.float64, device="cuda")
+    y = torch.empty_like(x)
+    torch.cuda.synchronize()
+    assert check(eye.data_ptr(), 33, x.data_ptr(), y.data_ptr(), 5, 1, 1, 0) == 0
+    # one product per result, one rounding of a 62-bit value
+    assert (y - x).abs().max() <= 2.0**-52 * x.abs().max()
