@@ -38,9 +38,13 @@ fdi_status launch_slice_transform(fdi_plan* p, const SliceMatrix& m, const doubl
 // and ny are at most kSmallN, the three z steps of the TPF in one when nz is.
 // Whole solves, digit products against small kernels (us): TPT 16^3 53.6 / 35.0,
 // 24^3 59.6 / 39.1, 32^3 61.6 / 45.3, 40^3 69.9 / 67.6; TPF 16^3 61.6 / 30.9, 32^3
-// 67.8 / 41.1, 40^3 78.0 / 67.8; 24 x 24 x 256 148 / 131 (several digit planes per
-// MMA since took 40^3 to 67.8 TPT and 74.0 TPF).  The plain multiply-adds
-// grow as n^4, so the line is drawn at 32.
+// 67.8 / 41.1, 40^3 78.0 / 67.8 (several digit planes per MMA since took 40^3 to
+// 67.8 TPT and 74.0 TPF, 32^3 to 57.5 / 43.2 and 63.6 / 39.1).  The plain
+// multiply-adds grow as n^4, so the line is drawn at 32.  It does not look at the
+// other extents, and fields with many planes of 32 x 32 cells or z columns of 32 lie
+// on the wrong side of it: TPT 16 x 16 x 256 111 / 94, 32 x 32 x 64 67.0 / 59.5, but
+// 32 x 32 x 128 86 / 90, 32 x 32 x 256 135 / 152; TPF 64 x 64 x 32 73.9 / 71.9, but
+// 128 x 128 x 32 127 / 144, 256 x 256 x 32 852 / 1056.
 constexpr int kSmallN = 32;
 bool small_plane_f64(const Field& f);
 bool small_z_f64(const Field& f);
